@@ -150,6 +150,13 @@ cudaError_t launch_bwd_f32(const float *q, const float *k, const float *v, const
 // fp32-input read on CUDA cores.
 cudaError_t launch_f32(const float *q, const float *k, const float *v, const float *beta, float *out, float *lse,
                        int B, int H, int T, int d, int causal, cudaStream_t stream);
+// The same read as 64-row by 64-key tiles of two fp32 contractions (fem_f32_tile.cu): d <= 128
+// (fp32 inputs) or d <= 32 (bf16), T <= kTileMaxT (query tiles are grid.y).
+constexpr int kTileMaxT = 64 * 65535;
+cudaError_t launch_tile_f32(const float *q, const float *k, const float *v, const float *beta, float *out, float *lse,
+                            int B, int H, int T, int d, int causal, cudaStream_t stream);
+cudaError_t launch_tile_bf16(const void *q, const void *k, const void *v, const float *beta, float *out, float *lse,
+                             int B, int H, int T, int d, int causal, cudaStream_t stream);
 // bf16 inputs of head dimension 16 or 32 on the same CUDA-core kernel (fp32 arithmetic).
 cudaError_t launch_simt_bf16(const void *q, const void *k, const void *v, const float *beta, float *out, float *lse,
                              int B, int H, int T, int d, int causal, cudaStream_t stream);

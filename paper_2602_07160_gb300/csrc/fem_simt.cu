@@ -1,7 +1,8 @@
 // The FEM read on CUDA cores, exact to fp32 rounding: fp32 inputs of any head
 // dimension up to 256, and bf16 inputs of head dimension 16 or 32 (too narrow
 // for the tensor-core read's 64-channel tiles to pay; here every product and
-// sum is fp32).
+// sum is fp32).  This kernel runs the shortest sequences and d > 128, the
+// tiles of fem_f32_tile.cu the others (use_tile below).
 //
 // One warp per output row t, four consecutive rows of one (b, h) per block;
 // lane l owns channels l, l+32, ...  The block stages the keys' K and V rows
@@ -249,13 +250,27 @@ static cudaError_t launch_simt(const In *q, const In *k, const In *v, const floa
   return cudaGetLastError();
 }
 
+// The tiled kernel (fem_f32_tile.cu) takes d up to max_d from 80 keys on, from 48 at d > 32 and from
+// 32 with at least 64 (b, h): its time hardly depends on the rows of a tile, this file's grows with
+// every row and key.  Measured, this kernel / the tiled one, causal, us: B*H = 1, d = 16: T 32 9.2 /
+// 12.5, T 64 13.3 / 12.5, T 96 18.2 / 14; B*H = 1, d = 64: T 32 13.7 / 13.7, T 64 22.2 / 15.9;
+// B*H = 16, d = 128: T 64 58.7 / 34.8; B*H = 64, d = 16: T 16 8.5 / 11, T 32 16.9 / 12; B*H = 384,
+// d = 64: T 8 14.6 / 36, T 32 103 / 37; B*H = 4, d = 64, T 2048: 2468 / 174.  bf16, B*H = 16, d = 32,
+// T 1024: 1271 / 56.
+static bool use_tile(int B, int H, int T, int d, int max_d) {
+  const bool long_enough = T >= 80 || (T >= 48 && d > 32) || (T >= 32 && static_cast<long long>(B) * H >= 64);
+  return d <= max_d && long_enough && T <= kTileMaxT;
+}
+
 cudaError_t launch_f32(const float *q, const float *k, const float *v, const float *beta, float *out, float *lse,
                        int B, int H, int T, int d, int causal, cudaStream_t stream) {
+  if (use_tile(B, H, T, d, 128)) return launch_tile_f32(q, k, v, beta, out, lse, B, H, T, d, causal, stream);
   return launch_simt<float>(q, k, v, beta, out, lse, B, H, T, d, causal, stream);
 }
 
 cudaError_t launch_simt_bf16(const void *q, const void *k, const void *v, const float *beta, float *out, float *lse,
                              int B, int H, int T, int d, int causal, cudaStream_t stream) {
+  if (use_tile(B, H, T, d, 32)) return launch_tile_bf16(q, k, v, beta, out, lse, B, H, T, d, causal, stream);
   return launch_simt<__nv_bfloat16>(static_cast<const __nv_bfloat16 *>(q), static_cast<const __nv_bfloat16 *>(k),
                                     static_cast<const __nv_bfloat16 *>(v), beta, out, lse, B, H, T, d, causal, stream);
 }
