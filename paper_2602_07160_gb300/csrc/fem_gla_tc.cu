@@ -334,13 +334,13 @@ __global__ void __launch_bounds__(256, 1)
       constexpr uint32_t id_s = idesc_f16(128, 128, true, false), id_n = idesc_f16(128, kGN, true, false);
 #pragma unroll
       for (int kk = 0; kk < kGM / 16; ++kk)
-        mma_f16_ss(tmem + kColS, smem_desc_sw128(sbase + GLay::kQ16 + kk * 32, 16, 1024),
+        mma_f16_ss(1u, tmem + kColS, smem_desc_sw128(sbase + GLay::kQ16 + kk * 32, 16, 1024),
                    smem_desc_sw128(sbase + GLay::kK16 + kk * 32, 16, 1024), id_s, kk > 0 ? 1u : 0u);
 #pragma unroll
       for (int kk = 0; kk < kGM / 16; ++kk)
-        mma_f16_ss(tmem + kColInter, smem_desc_sw128(sbase + GLay::kQ16 + kk * 32, 16, 1024),
+        mma_f16_ss(1u, tmem + kColInter, smem_desc_sw128(sbase + GLay::kQ16 + kk * 32, 16, 1024),
                    smem_desc_sw128(sbase + GLay::kS16 + kk * 32, 16, 1024), id_n, kk > 0 ? 1u : 0u);
-      mma_commit(bar_s);
+      mma_commit(1u, bar_s);
     }
     // ---- S o decay mask, as bf16 in A's 64 columns (thread = row of its warp's TMEM lane
     // quarter; warps 0-3 take keys 0..63, warps 4-7 keys 64..127)
@@ -377,15 +377,15 @@ __global__ void __launch_bounds__(256, 1)
       constexpr uint32_t id_n = idesc_f16(128, kGN, true, false);
 #pragma unroll
       for (int kk = 0; kk < kGC / 16; ++kk)
-        mma_f16_ts(tmem + kColIntra, tmem + kColA + kk * 8,
+        mma_f16_ts(1u, tmem + kColIntra, tmem + kColA + kk * 8,
                    smem_desc_sw128(sbase + GLay::kE16 + (kk >> 2) * GLay::kEBox + (kk & 3) * 32, 16, 1024), id_n,
                    kk > 0 ? 1u : 0u);
 #pragma unroll
       for (int kk = 0; kk < kGC / 16; ++kk)
-        mma_f16_ss(tmem + kColU, smem_desc_sw128(sbase + GLay::kKT16 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
+        mma_f16_ss(1u, tmem + kColU, smem_desc_sw128(sbase + GLay::kKT16 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
                    smem_desc_sw128(sbase + GLay::kE16 + (kk >> 2) * GLay::kEBox + (kk & 3) * 32, 16, 1024), id_n,
                    kk > 0 ? 1u : 0u);
-      mma_commit(bar_a);
+      mma_commit(1u, bar_a);
     }
     // ---- the outputs (thread = row of its warp's lane quarter; warps 4-7 take the CTA's channels
     // 0..15, warps 0-3 channels 16..31) and then the state (warps 0, 1, 4, 5, thread = feature)

@@ -127,30 +127,6 @@ enum : int {
   kBarSide = 33      // + side slot (8): tile k's rescale factors and moved-channel mask are in shared memory
 };
 
-
-__device__ __forceinline__ int pad_chunk(int n) { return (n + kFixChunk - 1) / kFixChunk * kFixChunk; }
-
-// Bounded wait that also gives up as soon as another role has given up.
-__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, unsigned *err, unsigned code,
-                                              volatile int *abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
-  while (true) {
-    if (mbar_try_wait_sleep(bar, parity, 200000u)) return true;
-    if (*abort_flag) return false;
-    if (global_timer_ns() - t0 > kWaitLimitNs) {
-      atomicOr(err, code);
-      *abort_flag = 1;
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
-  const __half2 v = __floats2half2_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&v);
-}
-
 __device__ __forceinline__ uint32_t pack_bf162(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&v);
@@ -178,7 +154,8 @@ __global__ void __launch_bounds__(384, 1)
   const uint32_t bars = sbase + Lay::kBar;
 #define FEM_BAR(i) (bars + 8u * static_cast<uint32_t>(i))
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // provably warp-uniform, like the warpgroup
   const int wg = __shfl_sync(0xffffffffu, tid >> 7, 0);  // warpgroup, provably warp-uniform
   const int n_qt = (T + kBlockQ - 1) / kBlockQ;
   const int n_kt_all = (T + kBlockK - 1) / kBlockK;
@@ -280,6 +257,10 @@ __global__ void __launch_bounds__(384, 1)
   // producer warps to the softmax (setmaxnreg) made the compiled code spill
   // more and ran slower.
   if (wg == 0) {
+  const uint32_t lead = lane == 0 ? 1u : 0u;
+  auto wait_warp = [&](int bar, int parity, unsigned code) {
+    return __all_sync(0xffffffffu, wait_or_abort(FEM_BAR(bar), parity, err, code, abort_flag)) != 0;
+  };
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA: Q and K
     if (lane == 0) {
@@ -303,65 +284,60 @@ __global__ void __launch_bounds__(384, 1)
       mbar_wait(FEM_BAR(kBarAccDone), 0, err, kErrWaitMma);
     }
   } else if (warp == 1) {
-    // ---------------------------------------------------------------- S issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc_qk = idesc_f16(128, 128, true, false);
-      bool ok = wait_or_abort(FEM_BAR(kBarQ), 0, err, kErrWaitTma, abort_flag);
-      for (int kt = 0; ok && kt < nk; ++kt) {
-        const int b = kt % kBufS, ks = kt % kStagesK;
-        const uint32_t use = static_cast<uint32_t>(kt / kBufS);
-        if (!(ok = wait_or_abort(FEM_BAR(kBarKFull + ks), (kt / kStagesK) & 1, err, kErrWaitTma, abort_flag))) break;
-        // the buffer's previous tile must have been consumed by its P E
-        if (use > 0 && !(ok = wait_or_abort(FEM_BAR(kBarPvDone + b), (use - 1) & 1, err, kErrWaitMma, abort_flag)))
+    // ---------------------------------------------------------------- S issuer (the warp converged,
+    // lane 0 issuing)
+    constexpr uint32_t idesc_qk = idesc_f16(128, 128, true, false);
+    bool ok = wait_warp(kBarQ, 0, kErrWaitTma);
+    for (int kt = 0; ok && kt < nk; ++kt) {
+      const int b = kt % kBufS, ks = kt % kStagesK;
+      const int use = kt / kBufS;
+      if (!(ok = wait_warp(kBarKFull + ks, (kt / kStagesK) & 1, kErrWaitTma))) break;
+      // the buffer's previous tile must have been consumed by its P E
+      if (use > 0 && !(ok = wait_warp(kBarPvDone + b, (use - 1) & 1, kErrWaitMma))) break;
+      tc_fence_after_sync();
+      const uint32_t sK = sbase + Lay::kK + ks * Lay::kTile;
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) {
+        const uint32_t off = (kk >> 2) * 16384 + (kk & 3) * 32;
+        mma_f16_ss(lead, tmem + b * 128, smem_desc_sw128(sbase + Lay::kQ + off, 16, 1024),
+                   smem_desc_sw128(sK + off, 16, 1024), idesc_qk, kk > 0 ? 1u : 0u);
+      }
+      mma_commit(lead, FEM_BAR(kBarSFull + b));
+      mma_commit(lead, FEM_BAR(kBarKEmpty + ks));
+    }
+    mma_commit(lead, FEM_BAR(kBarSDone));
+  } else if (warp == 2) {
+    // ---------------------------------------------------------------- PV issuer (likewise)
+    constexpr uint32_t idesc_pv = idesc_f16(128, D, ATTN, true);  // fp16 P and bank, or bf16 P and V
+    const uint32_t tAcc = tmem + Lay::kAccCol;
+    bool ok = true;
+    for (int kt = 0; ok && kt < nk; ++kt) {
+      const int b = kt % kBufS;
+      if (!(ok = wait_warp(kBarPFull + b, (kt / kBufS) & 1, kErrWaitMma))) break;
+      // each bank of the tile into its accumulator, D columns apart; the
+      // beta bank of a split diagonal tile into its own buffer
+#pragma unroll
+      for (int part = 0; part < kNB; ++part) {
+        const int e = kt * kNB + part, st = e % kSlotsE;
+        if (!(ok = wait_warp(kBarEFull + st, (e / kSlotsE) & 1, kErrWaitTma))) break;
+        const uint32_t sE = sbase + Lay::kE + st * Lay::kTile;
+        const bool to_diag = split && kt == nk - 1 && part == kNB - 1;
+        // the diagonal tile's buffer was last read by the P E of tile nk - kBufS
+        if (to_diag && nk >= kBufS &&
+            !(ok = wait_warp(kBarPvDone + nk % kBufS, ((nk - kBufS) / kBufS) & 1, kErrWaitMma)))
           break;
         tc_fence_after_sync();
-        const uint32_t sK = sbase + Lay::kK + ks * Lay::kTile;
+        const uint32_t dst = to_diag ? tDiag : tAcc + part * D;
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * 16384 + (kk & 3) * 32;
-          mma_f16_ss(tmem + b * 128, smem_desc_sw128(sbase + Lay::kQ + off, 16, 1024),
-                     smem_desc_sw128(sK + off, 16, 1024), idesc_qk, kk > 0 ? 1u : 0u);
-        }
-        mma_commit(FEM_BAR(kBarSFull + b));
-        mma_commit(FEM_BAR(kBarKEmpty + ks));
+        for (int kk = 0; kk < kBlockK / 16; ++kk)
+          mma_f16_ts(lead, dst, tmem + b * 128 + kk * 8, smem_desc_sw128(sE + kk * 2048, 16384, 1024), idesc_pv,
+                     ((kt > 0 && !to_diag) || kk > 0) ? 1u : 0u);
+        mma_commit(lead, FEM_BAR(kBarEEmpty + st));
       }
-      mma_commit(FEM_BAR(kBarSDone));
+      if (!ok) break;
+      mma_commit(lead, FEM_BAR(kBarPvDone + b));
     }
-  } else if (warp == 2) {
-    // ---------------------------------------------------------------- PV issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc_pv = idesc_f16(128, D, ATTN, true);  // fp16 P and bank, or bf16 P and V
-      const uint32_t tAcc = tmem + Lay::kAccCol;
-      bool ok = true;
-      for (int kt = 0; ok && kt < nk; ++kt) {
-        const int b = kt % kBufS;
-        if (!(ok = wait_or_abort(FEM_BAR(kBarPFull + b), (kt / kBufS) & 1, err, kErrWaitMma, abort_flag))) break;
-        // each bank of the tile into its accumulator, D columns apart; the
-        // beta bank of a split diagonal tile into its own buffer
-#pragma unroll
-        for (int part = 0; part < kNB; ++part) {
-          const int e = kt * kNB + part, st = e % kSlotsE;
-          if (!(ok = wait_or_abort(FEM_BAR(kBarEFull + st), (e / kSlotsE) & 1, err, kErrWaitTma, abort_flag))) break;
-          tc_fence_after_sync();
-          const uint32_t sE = sbase + Lay::kE + st * Lay::kTile;
-          const bool to_diag = split && kt == nk - 1 && part == kNB - 1;
-          // the diagonal tile's buffer was last read by the P E of tile nk - kBufS
-          if (to_diag && nk >= kBufS &&
-              !(ok = wait_or_abort(FEM_BAR(kBarPvDone + nk % kBufS), ((nk - kBufS) / kBufS) & 1, err, kErrWaitMma,
-                                   abort_flag)))
-            break;
-          const uint32_t dst = to_diag ? tDiag : tAcc + part * D;
-#pragma unroll
-          for (int kk = 0; kk < kBlockK / 16; ++kk)
-            mma_f16_ts(dst, tmem + b * 128 + kk * 8, smem_desc_sw128(sE + kk * 2048, 16384, 1024), idesc_pv,
-                       ((kt > 0 && !to_diag) || kk > 0) ? 1u : 0u);
-          mma_commit(FEM_BAR(kBarEEmpty + st));
-        }
-        if (!ok) break;
-        mma_commit(FEM_BAR(kBarPvDone + b));
-      }
-      mma_commit(FEM_BAR(kBarAccDone));  // completes once everything this thread issued is done
-    }
+    mma_commit(lead, FEM_BAR(kBarAccDone));  // completes once everything this warp issued is done
   }
   } else {
     // ---------------------------------------------------------------- softmax (warpgroup 1) or
