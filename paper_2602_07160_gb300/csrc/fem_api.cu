@@ -391,7 +391,7 @@ static int fwd_impl(const void *q, const void *k, const void *v, const float *be
   if (e == cudaSuccess && ev0) e = cudaEventRecord(ev0, s);
   if (e == cudaSuccess)
     e = launch_tc(d, tq, tk, te, ga ? &te0 : nullptr, out, beta, bw, lse, BH, H, T, causal, ga ? &gate : nullptr,
-                  ds->err, s, pdl);
+                  ds->err, ds->num_sms, s, pdl);
   if (e == cudaSuccess && ev1) e = cudaEventRecord(ev1, s);
   if (e == cudaSuccess)
     e = launch_fixup(q, k, v, beta, bw.chan, bw.shift, out, H, T, d, causal, bw.fixups, bw.fixup_count,

@@ -91,8 +91,13 @@ struct TcGate {
 // pdl: a programmatic dependent launch on the bank kernel before it.
 cudaError_t launch_tc(int d, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &te,
                       const CUtensorMap *te0, float *out, const float *beta, const BankWorkspace &w, float *lse,
-                      int BH, int H, int T, int causal, const TcGate *gate, unsigned *err, cudaStream_t stream,
-                      bool pdl = false);
+                      int BH, int H, int T, int causal, const TcGate *gate, unsigned *err, int num_sms,
+                      cudaStream_t stream, bool pdl = false);
+
+// The plain read at d = 64 with two CTAs per SM (fem_tc_half.cu); arguments and results as launch_tc.
+cudaError_t launch_tc_half(const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &te, float *out,
+                           const float *beta, const BankWorkspace &w, float *lse, int BH, int H, int T, int causal,
+                           unsigned *err, cudaStream_t stream, bool pdl);
 
 // The attention-mode comparator on the same kernel: o = softmax(q k^T / sqrt(d)) v
 // with bf16 P and V on the tensor cores (tv maps V like the bank).

@@ -898,8 +898,8 @@ static cudaError_t launch_tc_d(const CUtensorMap &tq, const CUtensorMap &tk, con
 
 cudaError_t launch_tc(int d, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &te,
                       const CUtensorMap *te0, float *out, const float *beta, const BankWorkspace &w, float *lse,
-                      int BH, int H, int T, int causal, const TcGate *gate, unsigned *err, cudaStream_t stream,
-                      bool pdl) {
+                      int BH, int H, int T, int causal, const TcGate *gate, unsigned *err, int num_sms,
+                      cudaStream_t stream, bool pdl) {
   const TcGate none = {nullptr, nullptr, nullptr, nullptr, nullptr};
   if ((te0 != nullptr) != (gate != nullptr)) return cudaErrorInvalidValue;
   if (gate) {
@@ -909,6 +909,13 @@ cudaError_t launch_tc(int d, const CUtensorMap &tq, const CUtensorMap &tk, const
       return launch_tc_d<128, true>(tq, tk, te, *te0, out, beta, w, lse, BH, H, T, causal, *gate, err, stream, pdl);
     return cudaErrorInvalidValue;
   }
+  // d = 64: two CTAs per SM (fem_tc_half.cu) once the grid holds more than one CTA per SM; with a CTA
+  // to itself on every SM this file's form is faster.  One / two per SM, us: B1 H1 T2048 causal (16 CTAs)
+  // 20.1 / 26.1, B1 H12 T1024 (96) 18.0 / 22.0, B1 H4 T4096 (128) 32.2 / 42.5, B8 H12 T512 (384) 31.4 /
+  // 29.3, B64 H6 T197 full (768) 43.6 / 29.3, B8 H12 T2048 (1536) 130.8 / 112.6.
+  const long long ctas = static_cast<long long>((T + kBlockQ - 1) / kBlockQ) * BH;
+  if (d == 64 && ctas > num_sms)
+    return launch_tc_half(tq, tk, te, out, beta, w, lse, BH, H, T, causal, err, stream, pdl);
   if (d == 64)
     return launch_tc_d<64, false>(tq, tk, te, te, out, beta, w, lse, BH, H, T, causal, none, err, stream, pdl);
   if (d == 128)
