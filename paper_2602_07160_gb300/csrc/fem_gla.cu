@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(32 * kGlaMaxWarps) gla_seg_kernel(
   const GlaLane L = gla_lane(beta, h, d);
   const size_t row0 = static_cast<size_t>(bh) * T;
   const int t_begin = p * seg_len, t_end = min(T, t_begin + seg_len);
-  float *st = state + ((static_cast<size_t>(bh) * n_seg + p) * blockDim.x + tid) * (MP + 1);
+  float *st = state + (static_cast<size_t>(bh) * n_seg + p) * (MP + 1) * blockDim.x + tid;  // float i at [i][thread]
   float S[MP];
   float lam = -INFINITY;  // log-scale of a beta > 0 channel's state
   if (MODE == 0) {
@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(32 * kGlaMaxWarps) gla_seg_kernel(
     for (int i = 0; i < MP; ++i) S[i] = 0.f;
   } else {
 #pragma unroll
-    for (int i = 0; i < MP; ++i) S[i] = st[i];
-    lam = st[MP];
+    for (int i = 0; i < MP; ++i) S[i] = st[i * blockDim.x];
+    lam = st[MP * blockDim.x];
   }
   float phi_acc = 0.f;
   // a stage's inputs by asynchronous 4-byte copies (any d), one commit group per stage
@@ -169,38 +169,51 @@ __global__ void __launch_bounds__(32 * kGlaMaxWarps) gla_seg_kernel(
   }
   if (MODE == 0) {
 #pragma unroll
-    for (int i = 0; i < MP; ++i) st[i] = S[i];
-    st[MP] = lam;
+    for (int i = 0; i < MP; ++i) st[i * blockDim.x] = S[i];
+    st[MP * blockDim.x] = lam;
     if (tid == 0) phi[static_cast<size_t>(bh) * n_seg + p] = phi_acc;
   }
 }
 
 // Start states in place of the local end states: start(0) = 0 and
-// start(p+1) = exp(Phi_p) start(p) + local_end(p), log-scaled for beta > 0.
+// start(p+1) = exp(Phi_p) start(p) + local_end(p), log-scaled for beta > 0.  A
+// warp per 32 lanes of a (b, h)'s blocks, each segment's state loaded while the
+// one before it is folded (a dependent load round a segment and states that lay
+// lane by lane took 107 us for 19 segments at B4 H4 m64 d128).
 template <int M>
-__global__ void __launch_bounds__(32 * kGlaMaxWarps) gla_combine_kernel(const float *__restrict__ beta, int H, int d,
-                                                                        int n_seg, float *__restrict__ state,
-                                                                        const float *__restrict__ phi) {
+__global__ void __launch_bounds__(32) gla_combine_kernel(const float *__restrict__ beta, int H, int d, int n_seg,
+                                                         float *__restrict__ state, const float *__restrict__ phi) {
   constexpr int MP = M / kGlaParts;
-  const int tid = threadIdx.x, bh = blockIdx.x, h = bh % H;
-  const GlaLane L = gla_lane(beta, h, d);
-  const bool scaled = L.real && !L.lin;
-  float R[MP];
+  const int warps = gridDim.x, threads = 32 * warps, bh = blockIdx.y, h = bh % H, lane = threadIdx.x;
+  const int j = blockIdx.x * kGlaChPerWarp + lane / kGlaParts;
+  const bool scaled = lane / kGlaParts != kGlaChPerWarp && j < d && beta[h * d + j] != 0.f;
+  float *st = state + static_cast<size_t>(bh) * n_seg * (MP + 1) * threads + blockIdx.x * 32 + lane;
+  const float *ph = phi + static_cast<size_t>(bh) * n_seg;
+  float R[MP], nx[MP + 1], nf = 0.f, rl = -INFINITY;
 #pragma unroll
   for (int i = 0; i < MP; ++i) R[i] = 0.f;
-  float rl = -INFINITY;
+  if (n_seg > 1) {  // the last segment's end state starts nothing
+#pragma unroll
+    for (int i = 0; i <= MP; ++i) nx[i] = st[static_cast<size_t>(i) * threads];
+    nf = ph[0];
+  }
   for (int p = 0; p < n_seg; ++p) {
-    float *st = state + ((static_cast<size_t>(bh) * n_seg + p) * blockDim.x + tid) * (MP + 1);
-    float loc[MP];
+    float loc[MP + 1];
+    const float f = nf;
 #pragma unroll
-    for (int i = 0; i < MP; ++i) loc[i] = st[i];
-    const float ll = st[MP];
+    for (int i = 0; i <= MP; ++i) loc[i] = nx[i];
+    float *here = st + static_cast<size_t>(p) * (MP + 1) * threads, *next = here + static_cast<size_t>(MP + 1) * threads;
+    if (p + 2 < n_seg) {
 #pragma unroll
-    for (int i = 0; i < MP; ++i) st[i] = R[i];
-    st[MP] = rl;
-    const float f = phi[static_cast<size_t>(bh) * n_seg + p];
+      for (int i = 0; i <= MP; ++i) nx[i] = next[static_cast<size_t>(i) * threads];
+      nf = ph[p + 1];
+    }
+#pragma unroll
+    for (int i = 0; i < MP; ++i) here[static_cast<size_t>(i) * threads] = R[i];
+    here[static_cast<size_t>(MP) * threads] = rl;
+    if (p + 1 == n_seg) break;
     if (scaled) {
-      const float lo = rl + f, ln = fmaxf(lo, ll);
+      const float ll = loc[MP], lo = rl + f, ln = fmaxf(lo, ll);
       if (ln == -INFINITY) continue;  // both still empty
       const float fr = expf(lo - ln), fl = expf(ll - ln);
 #pragma unroll
@@ -261,7 +274,7 @@ static cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v
   float *phi = state + (bytes / sizeof(float) - static_cast<size_t>(BH) * n_seg);
   const dim3 grid(n_seg, BH), block(32 * warps);
   gla_seg_kernel<M, 0><<<grid, block, 0, stream>>>(qf, kf, v, logdecay, beta, out, logz, H, T, d, seg_len, state, phi);
-  gla_combine_kernel<M><<<BH, block, 0, stream>>>(beta, H, d, n_seg, state, phi);
+  gla_combine_kernel<M><<<dim3(warps, BH), 32, 0, stream>>>(beta, H, d, n_seg, state, phi);
   gla_seg_kernel<M, 1><<<grid, block, 0, stream>>>(qf, kf, v, logdecay, beta, out, logz, H, T, d, seg_len, state, phi);
   return cudaGetLastError();
 }
