@@ -489,8 +489,18 @@ int fem_bwd_f32(const float *q, const float *k, const float *v, const float *bet
   if ((rc = device_state(&ds)) != FEM_OK) return rc;
   if ((rc = debug_check_beta(beta, static_cast<long long>(H) * d, ds, static_cast<cudaStream_t>(stream))) != FEM_OK)
     return rc;
-  return map_cuda(launch_bwd_f32(q, k, v, beta, out, lse, dout, dq, dk, dv, dbeta, B, H, T, d, causal,
-                                 static_cast<cudaStream_t>(stream)));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  void *ws = nullptr;
+  const size_t bytes = bwd_workspace_bytes(B, H, T, d);
+  if (bytes) {
+    cudaError_t e = ws_alloc(ds, &ws, bytes, s);
+    if (e != cudaSuccess) return map_cuda(e);
+  }
+  rc = map_cuda(launch_bwd_f32(q, k, v, beta, out, lse, dout, dq, dk, dv, dbeta, B, H, T, d, causal, ws, ds->num_sms, s));
+  if (!ws) return rc;
+  const cudaError_t e = cudaFreeAsync(ws, s);
+  if (rc != FEM_OK) return rc;
+  return map_cuda(e);
 }
 
 int fem_tdc_conv(const float *s, const float *u, float *h, int B, int T, int Hc, void *stream) {

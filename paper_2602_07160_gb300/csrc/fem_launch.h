@@ -147,10 +147,21 @@ cudaError_t launch_gla_tc(const float *qf, const float *kf, const float *v, cons
 size_t tdc_workspace_bytes(int B, int T, int Hc);
 cudaError_t launch_tdc(const float *s, const float *u, float *h, int B, int T, int Hc, void *ws, cudaStream_t stream);
 
-// Backward of the fp32 read (dq, dk, dv, and dbeta summed over batch and time).
+// Backward of the fp32 read (dq, dk, dv, and dbeta summed over batch and time): with ws
+// (bwd_workspace_bytes() bytes, not 0) as tiled contractions (fem_bwd_tile.cu), without it pair by
+// pair (fem_bwd.cu).
+size_t bwd_workspace_bytes(int B, int H, int T, int d);
 cudaError_t launch_bwd_f32(const float *q, const float *k, const float *v, const float *beta, const float *out,
                            const float *lse, const float *dout, float *dq, float *dk, float *dv, float *dbeta, int B,
-                           int H, int T, int d, int causal, cudaStream_t stream);
+                           int H, int T, int d, int causal, void *ws, int num_sms, cudaStream_t stream);
+cudaError_t launch_bwd_tile(const float *q, const float *k, const float *v, const float *beta, const float *out,
+                            const float *lse, const float *dout, float *dq, float *dk, float *dv, float *dbeta, int B,
+                            int H, int T, int d, int causal, void *ws, int num_sms, cudaStream_t stream);
+// Pair by pair; with peaked ([B H] marks) only the heads marked, their dbeta sums added to dbeta
+// [B H, d] instead of [H, d].
+cudaError_t launch_bwd_pairs(const float *q, const float *k, const float *v, const float *beta, const float *out,
+                             const float *lse, const float *dout, float *dq, float *dk, float *dv, float *dbeta, int B,
+                             int H, int T, int d, int causal, const int *peaked, cudaStream_t stream);
 
 // fp32-input read on CUDA cores.
 cudaError_t launch_f32(const float *q, const float *k, const float *v, const float *beta, float *out, float *lse,
