@@ -139,16 +139,32 @@ cudaError_t ws_alloc(DeviceState *ds, void **p, size_t bytes, cudaStream_t s) {
       props.location.type = cudaMemLocationTypeDevice;
       props.location.id = dev;
       cudaMemPool_t pool = nullptr;
-      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+      // no work on a stream, so it may also happen under a capture (a first call recorded into a graph)
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
+      e = cudaMemPoolCreate(&pool, &props);
       uint64_t keep = ~uint64_t(0);
-      if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      if (e == cudaSuccess && (e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess)
         cudaMemPoolDestroy(pool);
-        return e;
-      }
+      const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e != cudaSuccess) return e;
       ds->pool = pool;
+      if (back != cudaSuccess) return back;
     }
   }
   return cudaMallocFromPoolAsync(p, bytes, ds->pool, s);
+}
+
+// The same for a caller that has a form without a workspace: none (nullptr) for 0 bytes or where
+// there is no room, which is slower but not refused.
+cudaError_t ws_alloc_if(DeviceState *ds, void **p, size_t bytes, cudaStream_t s) {
+  *p = nullptr;
+  if (!bytes) return cudaSuccess;
+  const cudaError_t e = ws_alloc(ds, p, bytes, s);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  *p = nullptr;
+  return cudaSuccess;
 }
 
 // [BH, T, d] row-major tensor; boxes of box_rows rows x 128 bytes (64 16-bit
@@ -491,14 +507,11 @@ int fem_bwd_f32(const float *q, const float *k, const float *v, const float *bet
     return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   void *ws = nullptr;
-  const size_t bytes = bwd_workspace_bytes(B, H, T, d);
-  if (bytes) {
-    cudaError_t e = ws_alloc(ds, &ws, bytes, s);
-    if (e != cudaSuccess) return map_cuda(e);
-  }
+  cudaError_t e = ws_alloc_if(ds, &ws, bwd_workspace_bytes(B, H, T, d), s);
+  if (e != cudaSuccess) return map_cuda(e);
   rc = map_cuda(launch_bwd_f32(q, k, v, beta, out, lse, dout, dq, dk, dv, dbeta, B, H, T, d, causal, ws, ds->num_sms, s));
   if (!ws) return rc;
-  const cudaError_t e = cudaFreeAsync(ws, s);
+  e = cudaFreeAsync(ws, s);
   if (rc != FEM_OK) return rc;
   return map_cuda(e);
 }
