@@ -212,18 +212,20 @@ int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *l
 /*
  * fem_gla_fwd_tc -- the same read (fem_gla_fwd's definition and arguments)
  * chunked on the tensor cores, for m = d = 64 (FEM_ERR_UNSUPPORTED
- * otherwise).  One CTA per (b, h) walks 128-step chunks: the decay-masked
- * qf kf^T of the chunk against the chunk's value bank, qf against the state
- * of the earlier chunks, and the state's update, as bf16 contractions with
- * fp32 accumulation (tcgen05); the state itself is kept in fp32.  Channels
+ * otherwise), in chunks of 128 steps: the decay-masked qf kf^T of the chunk
+ * against the chunk's value bank, qf against the state of the earlier chunks,
+ * and the state's update, as bf16 contractions with fp32 accumulation
+ * (tcgen05); the state itself is kept in fp32.  Up to T = 256 a pair of CTAs
+ * per (b, h) walks the chunks; beyond, the chunks run in parallel around a scan
+ * of their states, with a workspace (at most 320 MB, or one head's 66 KB a
+ * chunk) allocated stream-ordered on `stream`.  Channels
  * with beta < 1/4 use the bank expm1(beta (v - c)) / beta anchored at the
- * smallest value so far, the others exp(beta v - lambda) with a log-scaled
+ * mean of the values so far, the others exp(beta v - lambda) with a log-scaled
  * state.  Accuracy is the bf16 read's for values of unit spread (max abs 2e-2,
  * mean abs 2e-3 against the float64 definition); per entry the bound is about
  * 2^-8 |v - c| (linear) or 2^-8 / beta (shifted), so it scales with the
  * values' spread.  Entries whose in-chunk part could be carried by terms
- * under fp32's range are recomputed exactly.  No workspace; qf, kf, v, out
- * 16-byte aligned.
+ * under fp32's range are recomputed exactly.  qf, kf, v, out 16-byte aligned.
  */
 int fem_gla_fwd_tc(const float *qf, const float *kf, const float *v, const float *logdecay,
                    const float *beta, float *out, float *logz, int B, int H, int T, int m, int d,

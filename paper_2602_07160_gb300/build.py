@@ -21,7 +21,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libfem.so")
-SOURCES = ["fem_api.cu", "fem_tc.cu", "fem_tc_half.cu", "fem_bank.cu", "fem_fixup.cu", "fem_simt.cu", "fem_f32_tile.cu", "fem_decode.cu", "fem_gla.cu", "fem_gla_tc.cu", "fem_tdc.cu", "fem_bwd.cu", "fem_bwd_tile.cu"]
+SOURCES = ["fem_api.cu", "fem_tc.cu", "fem_tc_half.cu", "fem_bank.cu", "fem_fixup.cu", "fem_simt.cu", "fem_f32_tile.cu", "fem_decode.cu", "fem_gla.cu", "fem_gla_tc.cu", "fem_gla_par.cu", "fem_tdc.cu", "fem_bwd.cu", "fem_bwd_tile.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

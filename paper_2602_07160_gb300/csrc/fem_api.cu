@@ -553,8 +553,15 @@ int fem_gla_fwd_tc(const float *qf, const float *kf, const float *v, const float
   if (rc != FEM_OK) return rc;
   if ((rc = debug_check_beta(beta, static_cast<long long>(H) * d, ds, static_cast<cudaStream_t>(stream))) != FEM_OK)
     return rc;
-  return map_cuda(launch_gla_tc(qf, kf, v, logdecay, beta, out, logz, B, H, T, ds->err,
-                                static_cast<cudaStream_t>(stream)));
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  void *ws = nullptr;
+  cudaError_t e = ws_alloc_if(ds, &ws, gla_par_workspace_bytes(B * H, T), s);
+  if (e != cudaSuccess) return map_cuda(e);
+  rc = map_cuda(launch_gla_tc(qf, kf, v, logdecay, beta, out, logz, B, H, T, ws, ds->err, s));
+  if (!ws) return rc;
+  e = cudaFreeAsync(ws, s);
+  if (rc != FEM_OK) return rc;
+  return map_cuda(e);
 }
 
 int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta, float *out,

@@ -5,6 +5,9 @@
 //   s_t(i) = K_{t,i} <qf_t, kf_i> (i <= t),  K_{t,i} = exp(g_{i+1} + ... + g_t),
 //   p_t = s_t / Z_t,  o_{t,j} = (1/beta_j) log sum_i p_t(i) exp(beta_j v_{i,j}).
 //
+// This form runs the shortest sequences, in one launch; from kGlaParMinChunks chunks on
+// their chunks run in parallel (fem_gla_par.cu).
+//
 // Two CTAs per (b, h), 32 value channels each, walk the sequence in chunks of
 // 128 steps (the score and mask work is repeated in both).  With gamma_t
 // the running sum of g inside the chunk (so K_{t,i} = exp(gamma_t - gamma_i) for
@@ -528,7 +531,8 @@ __global__ void __launch_bounds__(256, 1)
 }  // namespace
 
 cudaError_t launch_gla_tc(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
-                          float *out, float *logz, int B, int H, int T, unsigned *err, cudaStream_t stream) {
+                          float *out, float *logz, int B, int H, int T, void *ws, unsigned *err, cudaStream_t stream) {
+  if (ws) return launch_gla_par(qf, kf, v, logdecay, beta, out, logz, B, H, T, ws, err, stream);
   cudaError_t e = cudaFuncSetAttribute(gla_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GLay::kAlloc);
   if (e != cudaSuccess) return e;
   gla_tc_kernel<<<dim3(B * H, kVD / kGD), 256, GLay::kAlloc, stream>>>(qf, kf, v, logdecay, beta, out, logz, H, T,

@@ -137,9 +137,16 @@ cudaError_t launch_gla(const float *qf, const float *kf, const float *v, const f
                        float *out, float *logz, int BH, int H, int T, int m, int d, void *ws, int num_sms,
                        cudaStream_t stream);
 
-// The GLA-prior read chunked on the tensor cores (m = d = 64), one CTA per (b, h).
+// The GLA-prior read chunked on the tensor cores (m = d = 64): with ws (gla_par_workspace_bytes()
+// bytes, not 0) the chunks in parallel (fem_gla_par.cu), without it a CTA pair per (b, h) walking them
+// (fem_gla_tc.cu).  us, walking / parallel: B1 H1 T128 28 / 43, T300 47 / 44, T2048 226 / 43; B1 H12 T256
+// 42 / 46, T512 66 / 44; B16 H8 T100 46 / 50; B4 H16 T512 77 / 58, T8192 1069 / 365.
+constexpr int kGlaParMinChunks = 3;
+size_t gla_par_workspace_bytes(int BH, int T);
 cudaError_t launch_gla_tc(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
-                          float *out, float *logz, int B, int H, int T, unsigned *err, cudaStream_t stream);
+                          float *out, float *logz, int B, int H, int T, void *ws, unsigned *err, cudaStream_t stream);
+cudaError_t launch_gla_par(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
+                           float *out, float *logz, int B, int H, int T, void *ws, unsigned *err, cudaStream_t stream);
 
 // Time-decay conditioner convolution h_t = exp(-s_t) h_{t-1} + u_t over [B, T, Hc]
 // (segmented scan: one launch of 8-CTA clusters up to T = 16384, no workspace, then

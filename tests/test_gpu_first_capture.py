@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 CALLS = {
+    "gla_tc": "fem.fem_gla_fwd_tc(qf, qf, v, -0.1 * qf[..., 0].contiguous(), beta)",
     "backward": "fem.fem_bwd_f32(qf, qf, v, beta, out, lse, v)",
 }
 PROGRAM = """
