@@ -201,9 +201,10 @@ int fem_decode(const void *q, const void *k, const void *v, const float *beta, f
  *   logdecay : device, float32 [B, H, T], g_t <= 0
  *   beta     : device, float32 [H, d], beta >= 0 (0 = the prior mean)
  *   out      : device, float32 [B, H, T, d];  logz: device, float32 [B, H, T] or NULL
- * An O(T) recurrent scan in fp32 on CUDA cores, split into time segments
- * (segment end states, a combine over segments, then the outputs).  Allocates
- * its workspace (the segments' start states) stream-ordered on `stream`.
+ * In chunks of 64 steps, in fp32 on CUDA cores: each chunk's own state, the start
+ * states by a scan over chunks, then the outputs (one launch for T <= 64).
+ * Allocates its workspace (a state per chunk; at most 256 MB, heads and runs of
+ * chunks taken in turn beyond) stream-ordered on `stream`.
  */
 int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *logdecay,
                 const float *beta, float *out, float *logz, int B, int H, int T, int m, int d,

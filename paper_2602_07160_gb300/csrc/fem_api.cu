@@ -581,12 +581,19 @@ int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *l
   if (rc != FEM_OK) return rc;
   if ((rc = debug_check_beta(beta, static_cast<long long>(H) * d, ds, static_cast<cudaStream_t>(stream))) != FEM_OK)
     return rc;
-  const size_t bytes = gla_workspace_bytes(B * H, T, m, d, ds->num_sms, nullptr, nullptr);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   void *ws = nullptr;
-  cudaError_t e = ws_alloc(ds, &ws, bytes, s);
+  size_t cap = size_t(256) << 20;
+  size_t bytes = gla_workspace_bytes(B * H, T, m, d, cap);
+  cudaError_t e = ws_alloc_if(ds, &ws, bytes, s);
+  if (e == cudaSuccess && bytes && !ws) {  // little room: short runs of chunks
+    cap = size_t(1) << 20;
+    bytes = gla_workspace_bytes(B * H, T, m, d, cap);
+    e = ws_alloc(ds, &ws, bytes, s);
+  }
   if (e != cudaSuccess) return map_cuda(e);
-  rc = map_cuda(launch_gla(qf, kf, v, logdecay, beta, out, logz, B * H, H, T, m, d, ws, ds->num_sms, s));
+  rc = map_cuda(launch_gla(qf, kf, v, logdecay, beta, out, logz, B * H, H, T, m, d, cap, ws, s));
+  if (!ws) return rc;
   e = cudaFreeAsync(ws, s);
   if (rc != FEM_OK) return rc;
   return map_cuda(e);

@@ -9,284 +9,643 @@
 // attention state: o_{t,j} = (1/beta_j) log(<qf_t, S_{t,j}> / <qf_t, S_t>)
 // with S_{t,j} = sum_{i<=t} K_{t,i} kf_i exp(beta_j v_{i,j}), and the
 // normaliser Z_t = <qf_t, S_t>, S_t = sum_i K_{t,i} kf_i, is the same state for
-// a constant channel (the paper's "constant 1 channel").  A channel's state is
-// kept as exp(lam) S^ with the log-scale lam_t = max(lam_{t-1} + g_t,
-// beta v_{t,j}) -- the log of its largest term, which decays with the prior --
-// so neither exp(beta v) nor the decay under- or overflows (the per-channel
-// stabilisation of App. E); the normaliser's scale stays 0.  At beta_j = 0 the
+// a constant channel (the paper's "constant 1 channel").  At beta_j = 0 the
 // state carries v itself and o is the ratio (the prior mean).
 //
-// The scan is linear in the state, so the time axis is split into segments
-// (three passes): each segment's end state from a zero start, in parallel;
-// the segments' start states by a short sequential combine over segments,
-// start(p+1) = exp(Phi_p) start(p) + local_end(p) with Phi_p the segment's
-// summed log-decay (log-scaled like the states); then every segment again
-// from its start state, writing the outputs.  Within a segment four lanes
-// share a channel, each keeping a quarter of its m-float state in registers
-// (a warp holds 7 channels and the constant channel), and the block stages
-// qf, kf, g and v for kGlaSteps steps in shared memory, in two buffers filled
-// by asynchronous copies one stage ahead.  fp32 on CUDA cores.
+// In chunks of 64 steps, with gamma_t the running sum of g in the chunk, three
+// launches of fp32 contractions on CUDA cores (a lone chunk needs only the last):
+//
+//   local  U_j = sum_i kf_i exp(gamma_last - gamma_i + beta v_ij - lam'), the chunk's own state
+//   scan   the chunks in turn: start states, S' = exp(mu + gamma_last - mu') S + exp(lam' - mu') U
+//   out    in_t = sum_{i <= t} K_{t,i} <qf_t, kf_i> exp(beta v_i - lam), ix_t = <qf_t, S>, and the
+//          read of in_t e^lam + ix_t e^{mu + gamma_t} over Z_t, zi_t + exp(gamma_t) zx_t likewise
+//
+// Scales, so that neither exp(beta v) nor the decay under- or overflows (the per-channel
+// stabilisation of App. E): lam is the chunk's largest beta v, lam' its largest
+// beta v + gamma_last - gamma_i, and a state's log-scale mu the largest of its terms', decaying with
+// the prior; the normaliser's is 0.  lam may belong to a key that a row does not see: where in_t is
+// below 2^-90 of the row's in-chunk mass, or both parts together of the row's whole mass (fp32's
+// range could then hide terms that count), or not finite, the entry is read again key by key, from
+// the keys the row sees and the start state.  The decay's sums are taken in float64 and kept as
+// two floats, so a difference costs the rounding of its own size (steps of -60 are exact to 1e-7);
+// steps below kGlaFloor count as it: their weights are zero either way.
+//
+// What bounds it: instruction issue around the FMA pipe in out (three 64^3 contractions a chunk and
+// 64 channels), latency at the ends of a block.  B4 H4 T2048 m64 d128: local 24, scan 18, out 74 us, 120
+// in all, against 331 for a scan that walked segments of the sequence step by step, four lanes to a
+// channel's state (passes of 90 and 229 us, one dependent step at a time); B1 H1 T64 25 against 122,
+// B4 H16 T512 m16 d32 62 against 79.  Values of ten times unit spread with beta up to 100 send most
+// entries to the key-by-key read: 510 us at the first size.
 #include "fem_common.cuh"
+#include "fem_f32.cuh"
 #include "fem_launch.h"
 
 namespace fem {
+namespace {
 
-constexpr int kGlaSteps = 16;
-constexpr int kGlaParts = 4;                          // lanes per channel
-constexpr int kGlaChPerWarp = 32 / kGlaParts - 1;     // real channels per warp (the 8th is the normaliser)
-constexpr int kGlaMaxD = 155;
-constexpr int kGlaMaxWarps = (kGlaMaxD + kGlaChPerWarp - 1) / kGlaChPerWarp;
+constexpr int kSteps = 64, kCh = 64;  // steps of a chunk, channels of a block
+constexpr int kThreads = 256;         // thread (ty, tx): four rows (or features) against four keys (or channels)
+constexpr int kLd = kSteps + 4;       // leading dimension of the transposed Q and K tiles
+constexpr float kGlaGuard = 0x1p-90f;
+constexpr float kGlaFloor = -1e6f;
 
-__device__ __forceinline__ void cp_async4(float *dst, const float *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Per-lane role within a block of one (b, h).
-struct GlaLane {
-  int warp, lane, part, j;
-  bool real, lin;
-  float b;
+// Workspace of a group of heads and a run of chunks; per (head, chunk) unless noted.
+struct GlaWs {
+  float *u;      // [M][dp]: U, then the start state
+  float *z;      // [M]: the constant channel's
+  float *lam;    // [dp]: U's log-scale
+  float *mu;     // [dp]: the start state's
+  float *gl;     // the chunk's summed log-decay
+  float *carry;  // per head: [M][dp], [M] and [dp], the state (and mu) behind the run's last chunk
 };
 
-__device__ __forceinline__ GlaLane gla_lane(const float *beta, int h, int d) {
-  GlaLane L;
-  L.warp = threadIdx.x >> 5;
-  L.lane = threadIdx.x & 31;
-  const int cw = L.lane / kGlaParts;
-  L.part = L.lane % kGlaParts;
-  L.j = L.warp * kGlaChPerWarp + cw;
-  L.real = cw != kGlaChPerWarp && L.j < d;
-  L.b = L.real ? beta[h * d + L.j] : 0.f;
-  L.lin = L.b == 0.f;
-  return L;
+// gam[t] = g_0 + ... + g_t as a float pair (steps past the end add nothing); by warp 0.
+__device__ __forceinline__ void chunk_sums(const float *g, int rows, float2 *gam) {
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    float a = 2 * lane < rows ? g[2 * lane] : 0.f, b = 2 * lane + 1 < rows ? g[2 * lane + 1] : 0.f;
+    a = a < kGlaFloor ? kGlaFloor : a;
+    b = b < kGlaFloor ? kGlaFloor : b;
+    double s = static_cast<double>(a) + static_cast<double>(b);
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const double y = __shfl_up_sync(0xffffffffu, s, off);
+      if (lane >= off) s += y;
+    }
+    const double s0 = s - static_cast<double>(b);
+    const float h0 = static_cast<float>(s0), h1 = static_cast<float>(s);
+    gam[2 * lane] = make_float2(h0, static_cast<float>(s0 - static_cast<double>(h0)));
+    gam[2 * lane + 1] = make_float2(h1, static_cast<float>(s - static_cast<double>(h1)));
+  }
+}
+__device__ __forceinline__ float sum_diff(float2 a, float2 b) { return (a.x - b.x) + (a.y - b.y); }
+
+// The largest of x over the 16 row groups, per channel quad (thread = row group tid / 16, quad tid % 16).
+__device__ __forceinline__ float4 max_over_rows(float4 x, float4 (*red)[16]) {
+  const int q = threadIdx.x & 15;
+  red[threadIdx.x >> 4][q] = x;
+  __syncthreads();
+  float4 m = red[0][q];
+#pragma unroll
+  for (int p = 1; p < 16; ++p) {
+    const float4 y = red[p][q];
+    m = make_float4(fmaxf(m.x, y.x), fmaxf(m.y, y.y), fmaxf(m.z, y.z), fmaxf(m.w, y.w));
+  }
+  return m;
+}
+// a shift: 0 in place of -inf (no finite value), and for a linear channel
+__device__ __forceinline__ float shift_of(float m, float b) { return b > 0.f && m != -INFINITY ? m : 0.f; }
+
+__device__ __forceinline__ float4 beta4(const float *beta, int h, int d, int j) {
+  const float *p = beta + static_cast<size_t>(h) * d;
+  return make_float4(j < d ? p[j] : 0.f, j + 1 < d ? p[j + 1] : 0.f, j + 2 < d ? p[j + 2] : 0.f, j + 3 < d ? p[j + 3] : 0.f);
 }
 
-// MODE 0: the segment's end state from a zero start, and its summed log-decay.
-// MODE 1: the segment from its start state, writing out and log Z.
-template <int M, int MODE>
-__global__ void __launch_bounds__(32 * kGlaMaxWarps) gla_seg_kernel(
-    const float *__restrict__ qf, const float *__restrict__ kf, const float *__restrict__ v,
-    const float *__restrict__ logdecay, const float *__restrict__ beta, float *__restrict__ out,
-    float *__restrict__ logz, int H, int T, int d, int seg_len, float *__restrict__ state, float *__restrict__ phi) {
-  constexpr int MP = M / kGlaParts;  // state floats per lane
-  // the staged inputs in two buffers: the next stage's copies land while this one runs
-  __shared__ __align__(16) float s_q[2][kGlaSteps][M];
-  __shared__ __align__(16) float s_k[2][kGlaSteps][M];
-  __shared__ float s_v[2][kGlaSteps][kGlaMaxD];
-  __shared__ float s_g[2][kGlaSteps];
-  __shared__ float s_o[kGlaSteps][kGlaMaxD];
-  __shared__ float s_a[kGlaSteps], s_lz[kGlaSteps];
-  const int tid = threadIdx.x, p = blockIdx.x, n_seg = gridDim.x, bh = blockIdx.y, h = bh % H;
-  const GlaLane L = gla_lane(beta, h, d);
-  const size_t row0 = static_cast<size_t>(bh) * T;
-  const int t_begin = p * seg_len, t_end = min(T, t_begin + seg_len);
-  float *st = state + (static_cast<size_t>(bh) * n_seg + p) * (MP + 1) * blockDim.x + tid;  // float i at [i][thread]
-  float S[MP];
-  float lam = -INFINITY;  // log-scale of a beta > 0 channel's state
-  if (MODE == 0) {
+// ---------------------------------------------------------------------------
+// local: block per chunk and 64 channels.
+// ---------------------------------------------------------------------------
+template <int M>
+__global__ void __launch_bounds__(kThreads) gla_local_f32_kernel(const float *__restrict__ kf, const float *__restrict__ v,
+                                                                 const float *__restrict__ logdecay,
+                                                                 const float *__restrict__ beta, int h0, int H, int T,
+                                                                 int d, int dp, int c0, int nb, int vec, GlaWs w) {
+  constexpr int RT = M / 16;  // features of a thread
+  __shared__ __align__(16) float sK[kSteps * M], sE[kSteps * kCh];
+  __shared__ float4 red[16][16];
+  __shared__ float2 gam[kSteps];
+  __shared__ float s_dg[kSteps], s_z[4][M];
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, hd = blockIdx.z, j0 = blockIdx.y * kCh, jq = j0 + tx * 4;
+  const int c = c0 + blockIdx.x, rows = min(kSteps, T - c * kSteps);
+  const size_t r0 = static_cast<size_t>(h0 + hd) * T + static_cast<size_t>(c) * kSteps;
+  const size_t task = static_cast<size_t>(hd) * nb + blockIdx.x;
+  float4 x[4];
 #pragma unroll
-    for (int i = 0; i < MP; ++i) S[i] = 0.f;
-  } else {
-#pragma unroll
-    for (int i = 0; i < MP; ++i) S[i] = st[i * blockDim.x];
-    lam = st[MP * blockDim.x];
+  for (int u = 0; u < 4; ++u) {
+    const int r = ty + 16 * u;
+    x[u] = r < rows ? ld_row4(v + (r0 + r) * d, jq, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  float phi_acc = 0.f;
-  // a stage's inputs by asynchronous 4-byte copies (any d), one commit group per stage
-  auto stage = [&](int ts, int buf) {
-    const int ns = min(kGlaSteps, t_end - ts);
-    for (int e = tid; e < ns * M; e += blockDim.x) {
-      cp_async4(&s_q[buf][e / M][e % M], qf + (row0 + ts) * M + e);
-      cp_async4(&s_k[buf][e / M][e % M], kf + (row0 + ts) * M + e);
+#pragma unroll
+  for (int u = 0; u < M / 16; ++u) {
+    const int i = tid + u * kThreads;  // the chunk's rows of kf are contiguous
+    const float4 y = i * 4 < rows * M ? ld4(kf + r0 * M + i * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4 *>(sK + i * 4) = y;
+  }
+  chunk_sums(logdecay + r0, rows, gam);
+  __syncthreads();
+  if (tid < kSteps) s_dg[tid] = sum_diff(gam[kSteps - 1], gam[tid]);
+  if (tid == 0 && blockIdx.y == 0) w.gl[task] = gam[kSteps - 1].x;
+  __syncthreads();
+  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
+  float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  float4 y[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = ty + 16 * u;
+    const float g = s_dg[r];
+    y[u] = make_float4(fmaf(b.x, x[u].x, g), fmaf(b.y, x[u].y, g), fmaf(b.z, x[u].z, g), fmaf(b.w, x[u].w, g));
+    if (r < rows) m = make_float4(fmaxf(m.x, y[u].x), fmaxf(m.y, y[u].y), fmaxf(m.z, y[u].z), fmaxf(m.w, y[u].w));
+  }
+  m = max_over_rows(m, red);
+  if (ty == 0) *reinterpret_cast<float4 *>(w.lam + task * dp + jq) = m;
+  const float4 sh = make_float4(shift_of(m.x, b.x), shift_of(m.y, b.y), shift_of(m.z, b.z), shift_of(m.w, b.w));
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = ty + 16 * u;
+    const float dk = expf(s_dg[r]);
+    float4 e = make_float4(b.x > 0.f ? expf(y[u].x - sh.x) : x[u].x * dk, b.y > 0.f ? expf(y[u].y - sh.y) : x[u].y * dk,
+                           b.z > 0.f ? expf(y[u].z - sh.z) : x[u].z * dk, b.w > 0.f ? expf(y[u].w - sh.w) : x[u].w * dk);
+    if (r >= rows) e = make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4 *>(sE + r * kCh + tx * 4) = e;
+  }
+  __syncthreads();
+  float2 acc[RT][2];
+#pragma unroll
+  for (int r = 0; r < RT; ++r) acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+#pragma unroll 8
+  for (int i = 0; i < kSteps; ++i) {
+    const float4 e = ld4(sE + i * kCh + tx * 4);
+    float a[RT];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) a[r] = sK[i * M + ty * RT + r];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+      acc[r][0] = __ffma2_rn(make_float2(a[r], a[r]), make_float2(e.x, e.y), acc[r][0]);
+      acc[r][1] = __ffma2_rn(make_float2(a[r], a[r]), make_float2(e.z, e.w), acc[r][1]);
     }
-    for (int e = tid; e < ns * d; e += blockDim.x) cp_async4(&s_v[buf][e / d][e % d], v + (row0 + ts) * d + e);
-    for (int e = tid; e < ns; e += blockDim.x) cp_async4(&s_g[buf][e], logdecay + row0 + ts + e);
-    cp_async_commit();
+  }
+#pragma unroll
+  for (int r = 0; r < RT; ++r)
+    *reinterpret_cast<float4 *>(w.u + (task * M + ty * RT + r) * dp + jq) =
+        make_float4(acc[r][0].x, acc[r][0].y, acc[r][1].x, acc[r][1].y);
+  if (blockIdx.y == 0) {  // the constant channel, a quarter of the keys a thread
+    if (tid < 4 * M) {
+      const int f = tid % M, part = tid / M;
+      float z = 0.f;
+#pragma unroll
+      for (int i = 0; i < kSteps / 4; ++i) z = fmaf(sK[(part * (kSteps / 4) + i) * M + f], expf(s_dg[part * (kSteps / 4) + i]), z);
+      s_z[part][f] = z;
+    }
+    __syncthreads();
+    if (tid < M) w.z[task * M + tid] = (s_z[0][tid] + s_z[1][tid]) + (s_z[2][tid] + s_z[3][tid]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// scan: thread per state element (feature, channel; the constant channel's behind them), the run's
+// chunks in turn, the start states in U's place.  Bound by the states' bytes (from L2 at moderate
+// sizes); kAhead chunks' loads in flight, the scales' chain ahead of the exponentials.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) gla_scan_f32_kernel(const float *__restrict__ beta, int h0, int H, int d, int dp,
+                                                           int M, int first, int n, int nb, GlaWs w) {
+  constexpr int kAhead = 8;
+  const int i = blockIdx.x * 256 + threadIdx.x, hd = blockIdx.y;
+  if (i >= M * dp + M) return;
+  const bool is_z = i >= M * dp;
+  const int j = is_z ? 0 : i % dp;
+  if (!is_z && j >= d) return;
+  const size_t t0 = static_cast<size_t>(hd) * nb, stride = is_z ? M : static_cast<size_t>(M) * dp;
+  float *s = is_z ? w.z + t0 * M + (i - M * dp) : w.u + t0 * M * dp + i;
+  float *carry = w.carry + static_cast<size_t>(hd) * (M * dp + M + dp);
+  const bool scaled = !is_z && beta[static_cast<size_t>((h0 + hd) % H) * d + j] > 0.f, wr_mu = !is_z && i < dp;
+  float S = first ? 0.f : carry[i], mu = !scaled ? 0.f : first ? -INFINITY : carry[M * dp + M + j];
+  for (int c = 0; c < n; c += kAhead) {
+    float u[kAhead], lam[kAhead], gl[kAhead], fr[kAhead], fl[kAhead], at[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      const int p = min(c + q, n - 1);
+      u[q] = s[p * stride];
+      lam[q] = scaled ? w.lam[(t0 + p) * dp + j] : 0.f;
+      gl[q] = w.gl[t0 + p];
+    }
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      at[q] = mu;
+      const float eg = expf(gl[q]);
+      fr[q] = eg;
+      fl[q] = 1.f;
+      if (scaled && c + q < n) {
+        const float lo = mu + gl[q], to = fmaxf(lo, lam[q]);
+        const bool none = to == -INFINITY;  // no value yet
+        // exp(gl) apart, rounded as the constant channel's, unless it could underflow
+        fr[q] = none ? 0.f : gl[q] > -60.f ? eg * expf(mu - to) : expf(lo - to);
+        fl[q] = lam[q] == -INFINITY ? 0.f : expf(lam[q] - to);
+        mu = to;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      if (c + q >= n) break;
+      s[(c + q) * stride] = S;
+      if (wr_mu) w.mu[(t0 + c + q) * dp + j] = at[q];
+      S = fl[q] == 0.f ? fr[q] * S : fmaf(fr[q], S, fl[q] * u[q]);
+    }
+  }
+  carry[i] = S;
+  if (wr_mu) carry[M * dp + M + j] = mu;
+}
+
+// ---------------------------------------------------------------------------
+// out: block per chunk and 64 channels, about 70 KB of shared memory, three CTAs per SM.  Scores and
+// the state's part in one loop over the features; the masked weights take the state's place for the
+// in-chunk part, whose loop ends at a warp's last row.
+// ---------------------------------------------------------------------------
+template <int M>
+struct OutF32 {
+  static constexpr int kQ = 0, kK = M * kLd, kE = 2 * M * kLd, kS = kE + kSteps * kCh;
+  static constexpr int kFloats = kS + kSteps * kSteps;
+};
+
+template <int M>
+__global__ void __launch_bounds__(kThreads, 3)
+    gla_out_f32_kernel(const float *__restrict__ qf, const float *__restrict__ kf, const float *__restrict__ v,
+                       const float *__restrict__ logdecay, const float *__restrict__ beta, float *__restrict__ out,
+                       float *__restrict__ logz, int h0, int H, int T, int d, int dp, int c0, int nb, int vec, int vec_o,
+                       GlaWs w) {
+  using Lay = OutF32<M>;
+  extern __shared__ __align__(16) float gla_smem[];
+  float *sQ = gla_smem + Lay::kQ, *sK = gla_smem + Lay::kK, *sE = gla_smem + Lay::kE, *sS = gla_smem + Lay::kS, *sP = sS;
+  __shared__ float4 red[16][16];
+  __shared__ float2 gam[kSteps];
+  __shared__ float s_den[kSteps], s_sz[M];
+  __shared__ unsigned s_flag[kSteps][2];
+  const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 4, tx = tid & 15, hd = blockIdx.z, j0 = blockIdx.y * kCh, jq = j0 + tx * 4;
+  const int c = c0 + blockIdx.x, rows = min(kSteps, T - c * kSteps);
+  const size_t r0 = static_cast<size_t>(h0 + hd) * T + static_cast<size_t>(c) * kSteps;
+  const size_t task = static_cast<size_t>(hd) * nb + blockIdx.x;
+  const bool state = c > 0;
+  float4 x[4], qx[M / 16], kx[M / 16];
+#pragma unroll
+  for (int u = 0; u < M / 16; ++u) {  // lanes over rows: the transposed stores hit distinct banks
+    const int e = tid + u * kThreads, r = e % kSteps, f = (e / kSteps) * 4;
+    qx[u] = r < rows ? ld4(qf + (r0 + r) * M + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+    kx[u] = r < rows ? ld4(kf + (r0 + r) * M + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = ty + 16 * u;
+    x[u] = r < rows ? ld_row4(v + (r0 + r) * d, jq, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if (state) {
+#pragma unroll
+    for (int u = 0; u < M / 16; ++u) {
+      const int f = ty + 16 * u;
+      *reinterpret_cast<float4 *>(sS + f * kCh + tx * 4) = ld4(w.u + (task * M + f) * dp + jq);
+    }
+    if (tid < M) s_sz[tid] = w.z[task * M + tid];
+  }
+  if (tid < 2 * kSteps) s_flag[tid >> 1][tid & 1] = 0u;
+  chunk_sums(logdecay + r0, rows, gam);
+#pragma unroll
+  for (int u = 0; u < M / 16; ++u) {
+    const int e = tid + u * kThreads, r = e % kSteps, f = (e / kSteps) * 4;
+    sQ[f * kLd + r] = qx[u].x;
+    sQ[(f + 1) * kLd + r] = qx[u].y;
+    sQ[(f + 2) * kLd + r] = qx[u].z;
+    sQ[(f + 3) * kLd + r] = qx[u].w;
+    sK[f * kLd + r] = kx[u].x;
+    sK[(f + 1) * kLd + r] = kx[u].y;
+    sK[(f + 2) * kLd + r] = kx[u].z;
+    sK[(f + 3) * kLd + r] = kx[u].w;
+  }
+  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
+  float lam[4];
+  {
+    float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (ty + 16 * u < rows) m = make_float4(fmaxf(m.x, x[u].x), fmaxf(m.y, x[u].y), fmaxf(m.z, x[u].z), fmaxf(m.w, x[u].w));
+    m = max_over_rows(m, red);  // also: the tiles are written
+    lam[0] = shift_of(b.x * m.x, b.x);
+    lam[1] = shift_of(b.y * m.y, b.y);
+    lam[2] = shift_of(b.z * m.z, b.z);
+    lam[3] = shift_of(b.w * m.w, b.w);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int r = ty + 16 * u;
+    float4 e = make_float4(b.x > 0.f ? expf(fmaf(b.x, x[u].x, -lam[0])) : x[u].x,
+                           b.y > 0.f ? expf(fmaf(b.y, x[u].y, -lam[1])) : x[u].y,
+                           b.z > 0.f ? expf(fmaf(b.z, x[u].z, -lam[2])) : x[u].z,
+                           b.w > 0.f ? expf(fmaf(b.w, x[u].w, -lam[3])) : x[u].w);
+    if (r >= rows) e = make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4 *>(sE + r * kCh + tx * 4) = e;
+  }
+  // ---- scores (rows in packed pairs) and the state's part (channels in packed pairs)
+  float2 s[2][4], ix[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    s[0][i] = s[1][i] = make_float2(0.f, 0.f);
+    ix[i][0] = ix[i][1] = make_float2(0.f, 0.f);
+  }
+  const float *qp = sQ + ty * 4, *kp = sK + tx * 4, *sp = sS + tx * 4;
+  auto scores = [&](float4 a, float4 k4) {
+    const float2 ar[2] = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
+    const float kr[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s[0][i] = __ffma2_rn(ar[0], make_float2(kr[i], kr[i]), s[0][i]);
+      s[1][i] = __ffma2_rn(ar[1], make_float2(kr[i], kr[i]), s[1][i]);
+    }
   };
-  if (t_begin < t_end) stage(t_begin, 0);
-  int buf = 0;
-  for (int t0 = t_begin; t0 < t_end; t0 += kGlaSteps, buf ^= 1) {
-    const int n = min(kGlaSteps, t_end - t0);
-    // this stage's copies have landed, and every thread is done with the
-    // previous stage (whose buffer the next prefetch overwrites)
-    cp_async_wait_all();
-    __syncthreads();
-    if (t0 + kGlaSteps < t_end) stage(t0 + kGlaSteps, buf ^ 1);
-    for (int e = tid; e < n; e += blockDim.x) s_a[e] = expf(s_g[buf][e]);
-    __syncthreads();
-    for (int u = 0; u < n; ++u) {
-      const float x = L.real ? s_v[buf][u][L.j] : 0.f;
-      float E, a;
-      if (!L.real) {
-        E = 1.f;
-        a = s_a[u];
-      } else if (L.lin) {
-        E = x;
-        a = s_a[u];
-      } else {
-        const float le = L.b * x, lo = lam + s_g[buf][u];
-        const float ln = fmaxf(lo, le);
-        a = expf(lo - ln);  // 0 on the first step of a zero state
-        E = expf(le - ln);
-        lam = ln;
-      }
-      if (MODE == 0) phi_acc += s_g[buf][u];
-      const float4 *k4 = reinterpret_cast<const float4 *>(&s_k[buf][u][L.part * MP]);
-      const float4 *q4 = reinterpret_cast<const float4 *>(&s_q[buf][u][L.part * MP]);
-      float n0 = 0.f, n1 = 0.f;
+  auto rows_by_channels = [](float2 (&o)[4][2], float4 a, float4 e) {
+    const float ar[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
-      for (int i4 = 0; i4 < MP / 4; ++i4) {
-        const float4 kk = k4[i4];
-        S[4 * i4] = fmaf(a, S[4 * i4], E * kk.x);
-        S[4 * i4 + 1] = fmaf(a, S[4 * i4 + 1], E * kk.y);
-        S[4 * i4 + 2] = fmaf(a, S[4 * i4 + 2], E * kk.z);
-        S[4 * i4 + 3] = fmaf(a, S[4 * i4 + 3], E * kk.w);
-        if (MODE == 1) {
-          const float4 qq = q4[i4];
-          n0 = fmaf(qq.x, S[4 * i4], n0);
-          n1 = fmaf(qq.y, S[4 * i4 + 1], n1);
-          n0 = fmaf(qq.z, S[4 * i4 + 2], n0);
-          n1 = fmaf(qq.w, S[4 * i4 + 3], n1);
+    for (int i = 0; i < 4; ++i) {
+      o[i][0] = __ffma2_rn(make_float2(ar[i], ar[i]), make_float2(e.x, e.y), o[i][0]);
+      o[i][1] = __ffma2_rn(make_float2(ar[i], ar[i]), make_float2(e.z, e.w), o[i][1]);
+    }
+  };
+  if (state) {
+#pragma unroll 4
+    for (int f = 0; f < M; ++f) {
+      const float4 a = ld4(qp + f * kLd);
+      scores(a, ld4(kp + f * kLd));
+      rows_by_channels(ix, a, ld4(sp + f * kCh));
+    }
+  } else {
+#pragma unroll 8
+    for (int f = 0; f < M; ++f) scores(ld4(qp + f * kLd), ld4(kp + f * kLd));
+  }
+  // ---- the rows' masses (16 lanes share a row) and the masked weights
+  float zi[4], zx[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) zi[r] = zx[r] = 0.f;
+  if (state) {
+    for (int f = tx; f < M; f += 16) {
+      const float4 a = ld4(qp + f * kLd);
+      const float z = s_sz[f];
+      zx[0] = fmaf(a.x, z, zx[0]);
+      zx[1] = fmaf(a.y, z, zx[1]);
+      zx[2] = fmaf(a.z, z, zx[2]);
+      zx[3] = fmaf(a.w, z, zx[3]);
+    }
+  }
+  __syncthreads();  // the state's tile is consumed
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int key = tx * 4 + i;
+    const float2 gk = gam[key];
+    float p[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float sc = (r & 1) ? s[r >> 1][i].y : s[r >> 1][i].x;
+      p[r] = key <= ty * 4 + r ? sc * expf(sum_diff(gam[ty * 4 + r], gk)) : 0.f;
+      zi[r] += p[r];
+    }
+    *reinterpret_cast<float4 *>(sP + key * kSteps + ((ty ^ tx) << 2)) = make_float4(p[0], p[1], p[2], p[3]);
+  }
+#pragma unroll
+  for (int off = 8; off; off >>= 1)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      zi[r] += __shfl_xor_sync(0xffffffffu, zi[r], off);
+      zx[r] += __shfl_xor_sync(0xffffffffu, zx[r], off);
+    }
+  __syncthreads();
+  // ---- the in-chunk part
+  float2 in[4][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) in[i][0] = in[i][1] = make_float2(0.f, 0.f);
+  const int last = (tid >> 5) * 8 + 8;  // a warp's rows see no key from here on
+#pragma unroll 4
+  for (int i = 0; i < last; ++i)
+    rows_by_channels(in, ld4(sP + i * kSteps + ((ty ^ (i >> 2)) << 2)), ld4(sE + i * kCh + tx * 4));
+  // ---- the read
+  float mu[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) mu[q] = -INFINITY;
+  if (state) {
+    const float4 m4 = ld4(w.mu + task * dp + jq);
+    mu[0] = m4.x;
+    mu[1] = m4.y;
+    mu[2] = m4.z;
+    mu[3] = m4.w;
+  }
+  const float bj[4] = {b.x, b.y, b.z, b.w};
+  float rb[4], em[4];  // em: the state's scale over the chunk's, infinite where that overflows
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    rb[q] = bj[q] > 0.f ? 1.f / bj[q] : 0.f;
+    em[q] = mu[q] - lam[q] < 60.f ? expf(mu[q] - lam[q]) : INFINITY;
+  }
+  bool any = false;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int t = ty * 4 + r;
+    const float2 g2 = gam[t];
+    const float e0 = expf(g2.x), et = fmaf(e0, g2.y, e0), gt = g2.x + g2.y;
+    const float den = state ? fmaf(et, zx[r], zi[r]) : zi[r];
+    const float lo_in = kGlaGuard * zi[r], lo_sum = kGlaGuard * den, rden = 1.f / den;
+    unsigned flag = 0;
+    float o[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float a = (q & 1) ? in[r][q >> 1].y : in[r][q >> 1].x, y = (q & 1) ? ix[r][q >> 1].y : ix[r][q >> 1].x;
+      if (bj[q] > 0.f) {
+        // exp(gamma) apart, rounded as in the normaliser, unless it or the scales' ratio leaves fp32's range
+        float top = lam[q], sum = state ? fmaf(et * em[q], y, a) : a;
+        if (state && !(gt > -60.f && em[q] < INFINITY)) {
+          top = fmaxf(lam[q], mu[q] + gt);
+          sum = fmaf(a, expf(lam[q] - top), expf((mu[q] + gt) - top) * y);
         }
+        flag |= !(a >= lo_in) || !(sum >= lo_sum) ? 1u << q : 0u;
+        o[q] = (top + logf(sum * rden)) * rb[q];
+      } else {
+        flag |= !(fabsf(a) < INFINITY) ? 1u << q : 0u;
+        o[q] = (state ? fmaf(et, y, a) : a) * rden;
       }
-      if (MODE == 1) {
-        float num = n0 + n1;
+      if (jq + q >= d) flag &= ~(1u << q);
+    }
+    if (t < rows) {
+      float *orow = out + (r0 + t) * d + jq;
+      if (vec_o) {
+        if (jq < d) *reinterpret_cast<float4 *>(orow) = make_float4(o[0], o[1], o[2], o[3]);
+      } else {
 #pragma unroll
-        for (int off = 1; off < kGlaParts; off <<= 1) num += __shfl_xor_sync(0xffffffffu, num, off);
-        const float den = __shfl_sync(0xffffffffu, num, kGlaChPerWarp * kGlaParts);  // Z_t, the constant channel
-        if (L.real && L.part == 0) s_o[u][L.j] = L.lin ? num / den : (lam + (logf(num) - logf(den))) / L.b;
-        if (L.warp == 0 && L.lane == kGlaChPerWarp * kGlaParts) s_lz[u] = logf(den);
+        for (int q = 0; q < 4; ++q)
+          if (jq + q < d) orow[q] = o[q];
+      }
+      if (tx == 0) {
+        s_den[t] = den;
+        if (logz && blockIdx.y == 0) logz[r0 + t] = logf(den);
+      }
+      if (flag) {
+        atomicOr(&s_flag[t][tx >> 3], flag << ((tx & 7) * 4));
+        any = true;
       }
     }
-    if (MODE == 1) {
-      __syncthreads();  // the steps' outputs are in shared memory
-      for (int e = tid; e < n * d; e += blockDim.x) out[(row0 + t0) * d + e] = s_o[e / d][e % d];
-      if (logz)
-        for (int e = tid; e < n; e += blockDim.x) logz[row0 + t0 + e] = s_lz[e];
-    }
   }
-  if (MODE == 0) {
+  if (!__syncthreads_or(any)) return;
+  // ---- the flagged entries key by key, a warp per row.  The row's scores and decays once (lanes the keys
+  // lane and lane + 32 it sees), then for each 32 channels: lane = channel, the keys in turn, where four
+  // or more are flagged, else a channel at a time with the lanes over the keys.
+  float *s_sc = sP + (tid >> 5) * 2 * kSteps, *s_dg = s_sc + kSteps;  // the weights are consumed
+  const int t_end = min(rows, (tid >> 5) * 8 + 8);
+  for (int t = (tid >> 5) * 8; t < t_end; ++t) {
+    if (!(s_flag[t][0] | s_flag[t][1])) continue;
+    const float2 g2 = gam[t];
+    const float e0 = expf(g2.x), et = fmaf(e0, g2.y, e0), gt = g2.x + g2.y, den = s_den[t], lden = logf(den);
+    float sc[2], dg[2];
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < MP; ++i) st[i * blockDim.x] = S[i];
-    st[MP * blockDim.x] = lam;
-    if (tid == 0) phi[static_cast<size_t>(bh) * n_seg + p] = phi_acc;
+    for (int k2 = 0; k2 < 2; ++k2) {
+      const int i = lane + 32 * k2;
+      sc[k2] = 0.f;
+      dg[k2] = i <= t ? sum_diff(g2, gam[i]) : -INFINITY;
+      if (i <= t)
+        for (int f = 0; f < M; ++f) sc[k2] = fmaf(sQ[f * kLd + t], sK[f * kLd + i], sc[k2]);
+      s_sc[i] = sc[k2];
+      s_dg[i] = dg[k2];
+    }
+    __syncwarp();
+    // the read from the in-chunk sum acc at the shift m (linear: acc alone) and the state's part
+    auto read = [&](float bq, float m, float acc, float ixe, int j) {
+      if (!(bq > 0.f)) return (state ? fmaf(et, ixe, acc) : acc) / den;
+      const float la = acc == 0.f ? -INFINITY : m + logf(acc);
+      const float lb = ixe == 0.f ? -INFINITY : w.mu[task * dp + j] + gt + logf(ixe);
+      const float hi = fmaxf(la, lb), lo = fminf(la, lb);
+      const float ln = hi == -INFINITY ? hi : hi + log1pf(expf(lo - hi));
+      return ((la != la ? la : lb != lb ? lb : ln) - lden) / bq;
+    };
+    for (int half = 0; half < 2; ++half) {
+      unsigned fm = s_flag[t][half];
+      if (__popc(fm) >= 4) {
+        const int j = j0 + half * 32 + lane;
+        const bool on = (fm >> lane) & 1u;  // below d
+        const float bq = on ? beta[static_cast<size_t>((h0 + hd) % H) * d + j] : 0.f;
+        const float *vc = v + r0 * d + (on ? j : 0);
+        float m = -INFINITY, acc = 0.f, ixe = 0.f;
+        for (int i = 0; i <= t; ++i) m = fmaxf(m, fmaf(bq, __ldg(vc + static_cast<size_t>(i) * d), s_dg[i]));
+        for (int i = 0; i <= t; ++i) {
+          const float xv = __ldg(vc + static_cast<size_t>(i) * d), y = fmaf(bq, xv, s_dg[i]);
+          const float e = bq > 0.f ? expf(y - m) : expf(s_dg[i]) * xv;
+          if (!(bq > 0.f) || y != -INFINITY) acc = fmaf(s_sc[i], e, acc);
+        }
+        if (state && on)
+          for (int f = 0; f < M; ++f) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
+        if (on) out[(r0 + t) * d + j] = read(bq, m, acc, ixe, j);
+        continue;
+      }
+      while (fm) {
+        const int j = j0 + half * 32 + __ffs(fm) - 1;
+        fm &= fm - 1;
+        const float bq = beta[static_cast<size_t>((h0 + hd) % H) * d + j];
+        float y[2], m = -INFINITY, acc = 0.f, ixe = 0.f;
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2) {
+          const int i = lane + 32 * k2;
+          const float xv = i <= t ? __ldg(v + (r0 + i) * d + j) : 0.f;
+          y[k2] = i <= t ? fmaf(bq, xv, dg[k2]) : -INFINITY;
+          m = fmaxf(m, y[k2]);
+          if (!(bq > 0.f) && i <= t) acc = fmaf(sc[k2] * expf(dg[k2]), xv, acc);
+        }
+        if (state)
+          for (int f = lane; f < M; f += 32) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if (bq > 0.f) {
+#pragma unroll
+          for (int k2 = 0; k2 < 2; ++k2)
+            if (y[k2] != -INFINITY) acc = fmaf(sc[k2], expf(y[k2] - m), acc);
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) {
+          acc += __shfl_xor_sync(0xffffffffu, acc, off);
+          ixe += __shfl_xor_sync(0xffffffffu, ixe, off);
+        }
+        if (lane == 0) out[(r0 + t) * d + j] = read(bq, m, acc, ixe, j);
+      }
+    }
   }
 }
 
-// Start states in place of the local end states: start(0) = 0 and
-// start(p+1) = exp(Phi_p) start(p) + local_end(p), log-scaled for beta > 0.  A
-// warp per 32 lanes of a (b, h)'s blocks, each segment's state loaded while the
-// one before it is folded (a dependent load round a segment and states that lay
-// lane by lane took 107 us for 19 segments at B4 H4 m64 d128).
+size_t up64(size_t x) { return (x + 63) & ~size_t(63); }
+
+// Heads of a group, chunks of a run and the workspace's floats for at most `cap` bytes (one head and
+// eight chunks at least); none for a lone chunk.
+struct GlaPlan {
+  int heads, chunks;
+  size_t floats;
+};
+GlaPlan gla_plan(long long BH, int T, int m, int d, size_t cap, float *base, GlaWs *w) {
+  const int n_ch = (T + kSteps - 1) / kSteps, dp = (d + kCh - 1) / kCh * kCh;
+  if (n_ch == 1) return {static_cast<int>(BH < 65535 ? BH : 65535), 1, 0};
+  const size_t per = static_cast<size_t>(m) * dp + m + 2 * dp + 1, head = static_cast<size_t>(m) * dp + m + dp;
+  const size_t room = cap / sizeof(float) / per;
+  GlaPlan p;
+  if (room >= static_cast<size_t>(n_ch)) {
+    p.chunks = n_ch;
+    const long long fit = static_cast<long long>(cap / sizeof(float) / (per * n_ch + head));
+    p.heads = static_cast<int>(fit < 1 ? 1 : fit > 65535 ? 65535 : fit);
+    if (p.heads > BH) p.heads = static_cast<int>(BH);
+  } else {
+    p.heads = 1;
+    p.chunks = room < 8 ? 8 : static_cast<int>(room);
+    if (p.chunks > n_ch) p.chunks = n_ch;
+  }
+  const size_t n = static_cast<size_t>(p.heads) * p.chunks;
+  size_t o = 0;
+  auto take = [&](size_t count) {
+    float *q = base ? base + o : nullptr;
+    o += up64(count);
+    return q;
+  };
+  GlaWs l;
+  l.u = take(n * m * dp);
+  l.z = take(n * m);
+  l.lam = take(n * dp);
+  l.mu = take(n * dp);
+  l.gl = take(n);
+  l.carry = take(static_cast<size_t>(p.heads) * head);
+  p.floats = o;
+  if (w) *w = l;
+  return p;
+}
+
 template <int M>
-__global__ void __launch_bounds__(32) gla_combine_kernel(const float *__restrict__ beta, int H, int d, int n_seg,
-                                                         float *__restrict__ state, const float *__restrict__ phi) {
-  constexpr int MP = M / kGlaParts;
-  const int warps = gridDim.x, threads = 32 * warps, bh = blockIdx.y, h = bh % H, lane = threadIdx.x;
-  const int j = blockIdx.x * kGlaChPerWarp + lane / kGlaParts;
-  const bool scaled = lane / kGlaParts != kGlaChPerWarp && j < d && beta[h * d + j] != 0.f;
-  float *st = state + static_cast<size_t>(bh) * n_seg * (MP + 1) * threads + blockIdx.x * 32 + lane;
-  const float *ph = phi + static_cast<size_t>(bh) * n_seg;
-  float R[MP], nx[MP + 1], nf = 0.f, rl = -INFINITY;
-#pragma unroll
-  for (int i = 0; i < MP; ++i) R[i] = 0.f;
-  if (n_seg > 1) {  // the last segment's end state starts nothing
-#pragma unroll
-    for (int i = 0; i <= MP; ++i) nx[i] = st[static_cast<size_t>(i) * threads];
-    nf = ph[0];
-  }
-  for (int p = 0; p < n_seg; ++p) {
-    float loc[MP + 1];
-    const float f = nf;
-#pragma unroll
-    for (int i = 0; i <= MP; ++i) loc[i] = nx[i];
-    float *here = st + static_cast<size_t>(p) * (MP + 1) * threads, *next = here + static_cast<size_t>(MP + 1) * threads;
-    if (p + 2 < n_seg) {
-#pragma unroll
-      for (int i = 0; i <= MP; ++i) nx[i] = next[static_cast<size_t>(i) * threads];
-      nf = ph[p + 1];
-    }
-#pragma unroll
-    for (int i = 0; i < MP; ++i) here[static_cast<size_t>(i) * threads] = R[i];
-    here[static_cast<size_t>(MP) * threads] = rl;
-    if (p + 1 == n_seg) break;
-    if (scaled) {
-      const float ll = loc[MP], lo = rl + f, ln = fmaxf(lo, ll);
-      if (ln == -INFINITY) continue;  // both still empty
-      const float fr = expf(lo - ln), fl = expf(ll - ln);
-#pragma unroll
-      for (int i = 0; i < MP; ++i) R[i] = fmaf(fr, R[i], fl * loc[i]);
-      rl = ln;
-    } else {
-      const float fr = expf(f);
-#pragma unroll
-      for (int i = 0; i < MP; ++i) R[i] = fmaf(fr, R[i], loc[i]);
+cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
+                         float *out, float *logz, int BH, int H, int T, int d, size_t cap, void *ws, cudaStream_t stream) {
+  constexpr int kBytes = OutF32<M>::kFloats * 4;
+  cudaError_t e = cudaFuncSetAttribute(gla_out_f32_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+  if (e != cudaSuccess) return e;
+  GlaWs w = {};
+  const GlaPlan p = gla_plan(BH, T, M, d, cap, static_cast<float *>(ws), &w);
+  const int n_ch = (T + kSteps - 1) / kSteps, groups = (d + kCh - 1) / kCh, dp = groups * kCh;
+  const int vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(v) & 15u) == 0;
+  const int vec_o = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+  for (int h0 = 0; h0 < BH; h0 += p.heads) {
+    const int nh = BH - h0 < p.heads ? BH - h0 : p.heads;
+    for (int c0 = 0; c0 < n_ch; c0 += p.chunks) {
+      const int n = n_ch - c0 < p.chunks ? n_ch - c0 : p.chunks;
+      if (n_ch > 1) {
+        // the sequence's last chunk starts no other: what the scan reads in its slot goes nowhere
+        const int own = c0 + n == n_ch ? n - 1 : n;
+        if (own > 0)
+          gla_local_f32_kernel<M><<<dim3(own, groups, nh), kThreads, 0, stream>>>(kf, v, logdecay, beta, h0, H, T, d, dp,
+                                                                                  c0, p.chunks, vec, w);
+        gla_scan_f32_kernel<<<dim3((M * dp + M + 255) / 256, nh), 256, 0, stream>>>(beta, h0, H, d, dp, M, c0 == 0 ? 1 : 0,
+                                                                                    n, p.chunks, w);
+      }
+      gla_out_f32_kernel<M><<<dim3(n, groups, nh), kThreads, kBytes, stream>>>(qf, kf, v, logdecay, beta, out, logz, h0, H,
+                                                                               T, d, dp, c0, p.chunks, vec, vec_o, w);
     }
   }
-}
-
-// Resident blocks per SM of the output pass (the heavier of the two passes).
-static int gla_blocks_per_sm(int m, int threads) {
-  int n = 0;
-  cudaError_t e = cudaErrorInvalidValue;
-  if (m == 16) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gla_seg_kernel<16, 1>, threads, 0);
-  if (m == 32) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gla_seg_kernel<32, 1>, threads, 0);
-  if (m == 64) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, gla_seg_kernel<64, 1>, threads, 0);
-  return e == cudaSuccess && n > 0 ? n : 1;
-}
-
-size_t gla_workspace_bytes(int BH, int T, int m, int d, int num_sms, int *seg_len_out, int *n_seg_out) {
-  const int warps = (d + kGlaChPerWarp - 1) / kGlaChPerWarp;
-  // Segments of at least 64 steps.  A pass takes about (waves of resident
-  // blocks) x (segment length) steps of time, so the count minimises that
-  // product: whole waves of the grid, not a fraction of a last one.
-  const long long cap = static_cast<long long>(gla_blocks_per_sm(m, 32 * warps)) * num_sms;
-  const int max_seg = max(1, (T + 63) / 64);
-  int n_seg0 = 1;
-  long long best = -1;
-  for (int ns = 1; ns <= max_seg; ++ns) {
-    const long long waves = (static_cast<long long>(BH) * ns + cap - 1) / cap;
-    const long long cost = waves * ((T + ns - 1) / ns);
-    if (best < 0 || cost < best) {
-      best = cost;
-      n_seg0 = ns;
-    }
-    if (waves > 4) break;
-  }
-  const int seg_len = (T + n_seg0 - 1) / n_seg0;
-  const int n_seg = (T + seg_len - 1) / seg_len;
-  if (seg_len_out) *seg_len_out = seg_len;
-  if (n_seg_out) *n_seg_out = n_seg;
-  const size_t per_lane = static_cast<size_t>(m / kGlaParts + 1);
-  return (static_cast<size_t>(BH) * n_seg * 32 * warps * per_lane + static_cast<size_t>(BH) * n_seg) * sizeof(float);
-}
-
-template <int M>
-static cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v, const float *logdecay,
-                                const float *beta, float *out, float *logz, int BH, int H, int T, int d, void *ws,
-                                int num_sms, cudaStream_t stream) {
-  int seg_len = 0, n_seg = 0;
-  const int warps = (d + kGlaChPerWarp - 1) / kGlaChPerWarp;
-  const size_t bytes = gla_workspace_bytes(BH, T, M, d, num_sms, &seg_len, &n_seg);
-  float *state = static_cast<float *>(ws);
-  float *phi = state + (bytes / sizeof(float) - static_cast<size_t>(BH) * n_seg);
-  const dim3 grid(n_seg, BH), block(32 * warps);
-  gla_seg_kernel<M, 0><<<grid, block, 0, stream>>>(qf, kf, v, logdecay, beta, out, logz, H, T, d, seg_len, state, phi);
-  gla_combine_kernel<M><<<dim3(warps, BH), 32, 0, stream>>>(beta, H, d, n_seg, state, phi);
-  gla_seg_kernel<M, 1><<<grid, block, 0, stream>>>(qf, kf, v, logdecay, beta, out, logz, H, T, d, seg_len, state, phi);
   return cudaGetLastError();
 }
 
+}  // namespace
+
+size_t gla_workspace_bytes(int BH, int T, int m, int d, size_t cap) {
+  return gla_plan(BH, T, m, d, cap, nullptr, nullptr).floats * sizeof(float);
+}
+
 cudaError_t launch_gla(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
-                       float *out, float *logz, int BH, int H, int T, int m, int d, void *ws, int num_sms,
+                       float *out, float *logz, int BH, int H, int T, int m, int d, size_t cap, void *ws,
                        cudaStream_t stream) {
-  if (d > kGlaMaxD) return cudaErrorInvalidValue;
   switch (m) {
-    case 16: return launch_gla_m<16>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, ws, num_sms, stream);
-    case 32: return launch_gla_m<32>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, ws, num_sms, stream);
-    case 64: return launch_gla_m<64>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, ws, num_sms, stream);
+    case 16: return launch_gla_m<16>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, cap, ws, stream);
+    case 32: return launch_gla_m<32>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, cap, ws, stream);
+    case 64: return launch_gla_m<64>(qf, kf, v, logdecay, beta, out, logz, BH, H, T, d, cap, ws, stream);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -130,11 +130,12 @@ size_t decode_workspace_bytes(int BH, int T, int d, int num_sms);
 cudaError_t launch_decode(const CUtensorMap &tk, const void *q, const void *v, const float *beta, float *out,
                           float *lse, int BH, int H, int T, int d, float *part, unsigned *err, cudaStream_t stream);
 
-// FEM read over a GLA prior (fp32, segmented recurrent scan); m in {16, 32, 64},
-// d <= 155; `ws` holds gla_workspace_bytes() bytes (segment states).
-size_t gla_workspace_bytes(int BH, int T, int m, int d, int num_sms, int *seg_len, int *n_seg);
+// FEM read over a GLA prior (fp32, chunks of 64 steps around a scan of their states); m in {16, 32, 64};
+// `ws` holds gla_workspace_bytes() bytes for the same cap (0 for T <= 64): heads and runs of chunks are
+// taken in turn so that it stays within cap, or near 0.4 MB if that is more.
+size_t gla_workspace_bytes(int BH, int T, int m, int d, size_t cap);
 cudaError_t launch_gla(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
-                       float *out, float *logz, int BH, int H, int T, int m, int d, void *ws, int num_sms,
+                       float *out, float *logz, int BH, int H, int T, int m, int d, size_t cap, void *ws,
                        cudaStream_t stream);
 
 // The GLA-prior read chunked on the tensor cores (m = d = 64): with ws (gla_par_workspace_bytes()
