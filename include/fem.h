@@ -181,8 +181,9 @@ int fem_fwd_gated(const void *q, const void *k, const void *v, const float *beta
  *   out      : device, float32 [B, H, d];  lse: device, float32 [B, H] or NULL
  *   d in {64, 128}
  * Each CTA reads a chunk of 64 keys; the chunks' partials are merged with
- * log-add-exp in two levels, all in fp32 arithmetic.  Allocates a small
- * workspace (3d + 2 floats per chunk) stream-ordered on `stream`.
+ * log-add-exp, all in fp32 arithmetic: for the shorter caches inside one launch,
+ * else in two levels by a second one through a small workspace (3d + 2 floats
+ * per chunk) allocated stream-ordered on `stream`.
  */
 int fem_decode(const void *q, const void *k, const void *v, const float *beta, float *out,
                float *lse, int B, int H, int T, int d, void *stream);

@@ -615,17 +615,16 @@ int fem_decode(const void *q, const void *k, const void *v, const float *beta, f
   if ((rc = debug_check_beta(beta, static_cast<long long>(H) * d, ds, static_cast<cudaStream_t>(stream))) != FEM_OK)
     return rc;
   const int BH = B * H;
-  const size_t bytes = decode_workspace_bytes(BH, T, d, ds->num_sms);
+  const size_t bytes = decode_workspace_bytes(BH, T, d, ds->num_sms);  // 0: the one-launch form
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  void *ws = nullptr;
-  cudaError_t e = ws_alloc(ds, &ws, bytes, s);
-  if (e != cudaSuccess) return map_cuda(e);
   CUtensorMap tk;
-  if ((rc = make_map(&tk, k, BH, T, d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kDecodeKeysPerCta)) != FEM_OK) {
-    cudaFreeAsync(ws, s);
-    return rc;
-  }
-  rc = map_cuda(launch_decode(tk, q, v, beta, out, lse, BH, H, T, d, static_cast<float *>(ws), ds->err, s));
+  if ((rc = make_map(&tk, k, BH, T, d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, kDecodeKeysPerCta)) != FEM_OK) return rc;
+  void *ws = nullptr;
+  cudaError_t e = bytes ? ws_alloc(ds, &ws, bytes, s) : cudaSuccess;
+  if (e != cudaSuccess) return map_cuda(e);
+  rc = map_cuda(launch_decode(tk, q, v, beta, out, lse, BH, H, T, d, static_cast<float *>(ws), ds->num_sms,
+                              ds->err, s));
+  if (!ws) return rc;
   e = cudaFreeAsync(ws, s);
   if (rc != FEM_OK) return rc;
   return map_cuda(e);

@@ -122,13 +122,15 @@ cudaError_t launch_fixup(const void *q, const void *k, const void *v, const floa
 
 
 // Decode read of one query per (b, h) against T cached keys: per-CTA key-chunk
-// partials into `part` (decode_workspace_bytes), then their log-add-exp merge.
+// partials into `part` (decode_workspace_bytes), then their log-add-exp merge; in
+// one launch, with part null, where that is 0 (the shorter caches).
 // tk maps K as [BH, T, d] bf16 in boxes of kDecodeKeysPerCta rows x 64
 // channels with the 128-byte swizzle.
 constexpr int kDecodeKeysPerCta = 64;
 size_t decode_workspace_bytes(int BH, int T, int d, int num_sms);
 cudaError_t launch_decode(const CUtensorMap &tk, const void *q, const void *v, const float *beta, float *out,
-                          float *lse, int BH, int H, int T, int d, float *part, unsigned *err, cudaStream_t stream);
+                          float *lse, int BH, int H, int T, int d, float *part, int num_sms, unsigned *err,
+                          cudaStream_t stream);
 
 // FEM read over a GLA prior (fp32, chunks of 64 steps around a scan of their states); m in {16, 32, 64};
 // `ws` holds gla_workspace_bytes() bytes for the same cap (0 for T <= 64): heads and runs of chunks are
