@@ -172,6 +172,8 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 // stream still runs; it waits here, before touching any global memory that
 // kernel (or one before it) writes or reads, for that kernel's completion and
 // the visibility of its writes.  Without the attribute the wait returns at once.
+// Such memory is not read through a const __restrict__ parameter: the compiler
+// takes that as constant over the whole kernel and may load it before the wait.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream be scheduled once every block of this one
 // has started (or passed here): its blocks then take the SMs this kernel's tail

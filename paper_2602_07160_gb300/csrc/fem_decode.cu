@@ -414,8 +414,8 @@ __global__ void __launch_bounds__(kDecThreads) decode_cluster_kernel(const __gri
 constexpr int kDecMergeGroups = 8;
 
 template <int D>
-__global__ void __launch_bounds__(D) decode_merge_kernel(const float *__restrict__ part, int n_parts,
-                                                         float *__restrict__ gpart, int *__restrict__ count,
+__global__ void __launch_bounds__(D) decode_merge_kernel(const float *part, int n_parts,
+                                                         float *gpart, int *__restrict__ count,
                                                          const float *__restrict__ beta, int H,
                                                          float *__restrict__ out, float *__restrict__ lse) {
   constexpr int G = kDecMergeGroups, F = DecPart<D>::kFloats;
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(D) decode_merge_kernel(const float *__restrict
   if (grp >= n_groups) return;
   // launched as a programmatic dependent of the chunk kernel: its partials
   // are complete and visible once this wait returns
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_dep_wait();
   float r[5];
   dec_fold_range<D>(part + static_cast<size_t>(bh) * n_parts * F, grp * n_parts / n_groups,
                     (grp + 1) * n_parts / n_groups, j, b, inv_b, r);

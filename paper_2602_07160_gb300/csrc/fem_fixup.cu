@@ -145,6 +145,7 @@ __device__ __forceinline__ void fold_tile(float &c, float &A, float &W, float L,
   W += W2;
 }
 
+// What the launches before this one wrote comes by pointers that are not __restrict__ (see grid_dep_wait).
 // SPLIT: long recomputations go over key-tile segments (part != null); otherwise
 // every chunk runs whole and the kernel carries none of that machinery.
 template <int D, bool SPLIT>
@@ -152,12 +153,12 @@ __global__ void __launch_bounds__(kFixThreads, D == 64 ? 4 : 3) fixup_kernel(con
                                                             const __nv_bfloat16 *__restrict__ k,
                                                             const __nv_bfloat16 *__restrict__ v,
                                                             const float *__restrict__ beta,
-                                                            const ChanInfo *__restrict__ chan,
-                                                            const float *__restrict__ shift, float *__restrict__ out,
+                                                            const ChanInfo *chan,
+                                                            const float *shift, float *__restrict__ out,
                                                             int H, int T, int causal,
-                                                            const FixupEntry *__restrict__ entries,
-                                                            const int *__restrict__ count,
-                                                            const int *__restrict__ rows_listed,
+                                                            const FixupEntry *entries,
+                                                            const int *count,
+                                                            const int *rows_listed,
                                                             int *__restrict__ next_chunk,
                                                             int *__restrict__ last_rows, TcGate gate,
                                                             int *__restrict__ fix_long, FixSlot *__restrict__ slots,
@@ -174,7 +175,8 @@ __global__ void __launch_bounds__(kFixThreads, D == 64 ? 4 : 3) fixup_kernel(con
   __shared__ float sS[kFixChunk][kBlockK];  // the chunk's scores (log2 units), then the tile's P
   __shared__ int s_ch, s_slot, s_seg, s_merge, s_split;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_chunks = *count / kFixChunk;
+  // thread 0 alone knows the list's length: every warp leaves the loop below on the same s_ch
+  const int n_chunks = tid == 0 ? __ldcg(count) / kFixChunk : 0;
   if (blockIdx.x == 0 && tid == 0 && last_rows) *last_rows = *rows_listed;
   const float scale = kLog2e * rsqrtf(static_cast<float>(D));
   const int n_kt = (T + kBlockK - 1) / kBlockK;
@@ -184,20 +186,20 @@ __global__ void __launch_bounds__(kFixThreads, D == 64 ? 4 : 3) fixup_kernel(con
 
   // warp 0 claims the work; lane 0 keeps the list's next chunk claimed one ahead and the
   // chunk this block split
-  int claim = n_chunks, my_slot = -1, my_nseg = 0, my_chunk = 0;
+  int claim = 0, my_slot = -1, my_nseg = 0, my_chunk = 0;
   if (tid == 0) claim = atomicAdd(next_chunk, 1);
   for (;;) {
     // the next piece: (1) the next segment of the chunk this block split; (2) the list's
     // next chunk; (3) once the list is exhausted, a segment of a chunk another block split
     if (!SPLIT) {
       if (tid == 0) {
-        s_ch = claim;
+        s_ch = claim < n_chunks ? claim : -1;
         s_slot = -1;
         s_seg = 0;
         if (claim < n_chunks) claim = atomicAdd(next_chunk, 1);
       }
     } else if (warp == 0) {
-      int ch = n_chunks, slot = -1, seg = 0;
+      int ch = -1, slot = -1, seg = 0;
       if (lane == 0) {
         if (my_slot >= 0) {
           const int sg = atomicAdd(&slots[my_slot].next, 1);
@@ -217,7 +219,7 @@ __global__ void __launch_bounds__(kFixThreads, D == 64 ? 4 : 3) fixup_kernel(con
       ch = __shfl_sync(0xffffffffu, ch, 0);
       slot = __shfl_sync(0xffffffffu, slot, 0);
       seg = __shfl_sync(0xffffffffu, seg, 0);
-      if (slot < 0 && ch >= n_chunks) {
+      if (slot < 0 && ch < 0) {
         // lanes over the slots, 32 at a time; the lowest lane holding one with segments left claims
         const int nl = min(*reinterpret_cast<volatile int *>(fix_long), kFixPoolSlots);
         for (int b0 = 0; b0 < nl && slot < 0; b0 += 32) {
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(kFixThreads, D == 64 ? 4 : 3) fixup_kernel(con
     __syncthreads();
     const int ch = s_ch;
     int slot = SPLIT ? s_slot : -1, seg = SPLIT ? s_seg : 0;
-    if (ch >= n_chunks) break;
+    if (ch < 0) break;  // nothing left
     const FixupEntry ent = entries[ch * kFixChunk + warp];
     const FixupEntry ent0 = entries[ch * kFixChunk];  // the chunk's first entry is a real row
     const int bh = ent0.row / T, h = bh % H;
