@@ -347,11 +347,11 @@ static BankWorkspace bank_workspace(uint8_t *ws, const WsLayout &w) {
   return bw;
 }
 
-// Gated part of a read: the mean's pre-pass workspace (ws_layout, non-causal)
-// and its zero beta, the gates, and mu_side (the mean at the fix-up entries).
+// Gated part of a read: the mean's pre-pass workspace (ws_layout, non-causal),
+// the gates, and mu_side (the mean at the fix-up entries).
 struct GatedArgs {
   uint8_t *ws0;
-  const float *zero_beta, *lam, *g;
+  const float *lam, *g;
   float *mu_side;
 };
 
@@ -392,12 +392,10 @@ static int fwd_impl(const void *q, const void *k, const void *v, const float *be
 
   // the four counters, and the split slots when the fix-up may split
   cudaError_t e = cudaMemsetAsync(bw.fixup_count, 0, bw.fix_part ? kCountBytes : 4 * sizeof(int), s);
-  // the mean's bank (every channel linear at beta = 0: v - c with c the channel mean)
-  if (e == cudaSuccess && ga)
-    e = launch_value_bank(v, tv, te0, ga->zero_beta, BH, H, T, d, bw0, ds->err, ds->num_sms, s);
-  if (ga) bw.tstat = bw0.tstat;  // the tiles' statistics do not depend on beta
+  // gated: also the mean's bank (every channel linear at beta = 0: v - c with c the channel mean)
   if (e == cudaSuccess)
-    e = launch_value_bank(v, tv, te, beta, BH, H, T, d, bw, ds->err, ds->num_sms, s, ga != nullptr);
+    e = launch_value_bank(v, tv, te, ga ? &te0 : nullptr, beta, BH, H, T, d, bw, ga ? &bw0 : nullptr, ds->err,
+                          ds->num_sms, s);
   const cudaEvent_t ev0 = t_ev_start, ev1 = t_ev_stop;
   t_ev_start = t_ev_stop = nullptr;
   // the read and the fix-up are programmatic dependent launches on the kernel before them (their
@@ -463,28 +461,23 @@ int fem_fwd_gated(const void *q, const void *k, const void *v, const float *beta
   if ((rc = device_state(&ds)) != FEM_OK) return rc;
   if ((rc = debug_check_beta(beta_max, static_cast<long long>(H) * d, ds, static_cast<cudaStream_t>(stream))) != FEM_OK)
     return rc;
-  // workspace: the beta_max read's, the mean's pre-pass (non-causal layout),
-  // a zero beta [H, d], and mu_side [B, H, T, d] fp32 for the fix-up's entries
-  // (the guard can list entries of either mask)
+  // workspace: the beta_max read's, the mean's pre-pass (non-causal layout), and
+  // mu_side [B, H, T, d] fp32 for the fix-up's entries (the guard can list entries of either mask)
   const size_t n = static_cast<size_t>(B) * H * T * d;
   const size_t ws_bytes = round256(fem_fwd_workspace_bytes(B, H, T, d, causal));
   const size_t ws0_bytes = round256(fem_fwd_workspace_bytes(B, H, T, d, 0));
-  const size_t zb_bytes = round256(static_cast<size_t>(H) * d * sizeof(float));
   const size_t mu_bytes = round256(n * sizeof(float));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   void *buf = nullptr;
-  cudaError_t e = ws_alloc(ds, &buf, ws_bytes + ws0_bytes + zb_bytes + mu_bytes, s);
+  cudaError_t e = ws_alloc(ds, &buf, ws_bytes + ws0_bytes + mu_bytes, s);
   if (e != cudaSuccess) return map_cuda(e);
   uint8_t *p = static_cast<uint8_t *>(buf);
   GatedArgs ga;
   ga.ws0 = p + ws_bytes;
-  ga.zero_beta = reinterpret_cast<const float *>(p + ws_bytes + ws0_bytes);
   ga.lam = lam;
   ga.g = gate;
-  ga.mu_side = reinterpret_cast<float *>(p + ws_bytes + ws0_bytes + zb_bytes);
-  e = cudaMemsetAsync(const_cast<float *>(ga.zero_beta), 0, static_cast<size_t>(H) * d * sizeof(float), s);
-  rc = map_cuda(e);
-  if (rc == FEM_OK) rc = fwd_impl(q, k, v, beta_max, out, lse, B, H, T, d, causal, p, &ga, ds, s);
+  ga.mu_side = reinterpret_cast<float *>(p + ws_bytes + ws0_bytes);
+  rc = fwd_impl(q, k, v, beta_max, out, lse, B, H, T, d, causal, p, &ga, ds, s);
   e = cudaFreeAsync(buf, s);
   if (rc != FEM_OK) return rc;
   return map_cuda(e);

@@ -157,11 +157,27 @@ __device__ __forceinline__ float4 bank_coef(bool lin, float b, float c) {
 // parallel.  Besides the schedule it writes the bank's per-tile coefficients
 // (BankCoef) and the moved-channel word of its group.
 // ---------------------------------------------------------------------------
+// A read's plan and bank; beta null is beta = 0 (the prior mean).  The gated read makes two of the same
+// V, as grid z = 0 and 1 here and as alternate tasks of the bank kernel (two plans and two banks in turn,
+// each 7 to 8 us at B4 H4 T2048 d128 and far from filling the chip, made that call 118 us; it is 106 now).
+struct BankSet {
+  const float *beta;
+  ChanInfo *chan;
+  float *shift, *rfac;
+  unsigned *colmask;
+  float4 *bcoef;
+  float *colsum;
+};
+
 template <int D>
-__global__ void __launch_bounds__(128) plan_kernel(const float4 *__restrict__ tstat, const float *__restrict__ beta,
-                                                   int H, int T, int n_kt, ChanInfo *__restrict__ chan,
-                                                   float *__restrict__ shift, float *__restrict__ rfac,
-                                                   unsigned *__restrict__ colmask, float4 *__restrict__ bcoef) {
+__global__ void __launch_bounds__(128) plan_kernel(const float4 *__restrict__ tstat, const BankSet set0,
+                                                   const BankSet set1, int H, int T, int n_kt) {
+  const BankSet set = blockIdx.z ? set1 : set0;
+  const float *beta = set.beta;
+  ChanInfo *__restrict__ chan = set.chan;
+  float *__restrict__ shift = set.shift, *__restrict__ rfac = set.rfac;
+  unsigned *__restrict__ colmask = set.colmask;
+  float4 *__restrict__ bcoef = set.bcoef;
   constexpr int kParts = 4, kPer = 16, kWin = kParts * kPer;
   __shared__ unsigned s_mask[kWin];
   __shared__ float s_tm[kWin][33];      // the window's tile maxima per channel of the block
@@ -169,7 +185,7 @@ __global__ void __launch_bounds__(128) plan_kernel(const float4 *__restrict__ ts
   const int tid = threadIdx.x, part = tid % kParts, lane = tid & 31;
   const int grp = blockIdx.y, j = grp * 32 + tid / kParts;
   const int bh = blockIdx.x, h = bh % H;
-  const float b = beta[h * D + j];
+  const float b = beta ? beta[h * D + j] : 0.f;
   const float4 *ts = tstat + static_cast<size_t>(bh) * n_kt * D + j;
   // pass 1: the channel's max, min and sum over every key tile
   float gmax = -INFINITY, gmin = INFINITY, gsum = 0.f;
@@ -357,10 +373,12 @@ __device__ __forceinline__ void bank_entries4(const float4 cf, const float (&x)[
 
 template <int D>
 __global__ void __launch_bounds__(256, 2) bank_kernel(const __grid_constant__ CUtensorMap tv,
-                                                       const __grid_constant__ CUtensorMap te,
-                                                       const float4 *__restrict__ bcoef, int T, int n_kt,
-                                                       int n_tiles, int reverse, float *__restrict__ colsum,
-                                                       unsigned *__restrict__ err) {
+                                                       const __grid_constant__ CUtensorMap te0,
+                                                       const __grid_constant__ CUtensorMap te1,
+                                                       const float4 *__restrict__ bcoef0,
+                                                       const float4 *__restrict__ bcoef1, int sets, int T, int n_kt,
+                                                       int n_tiles, int reverse, float *__restrict__ colsum0,
+                                                       float *__restrict__ colsum1, unsigned *__restrict__ err) {
   using M = BankMap<D>;
   // the read kernel, a programmatic dependent launch, may take the SMs this pass's tail leaves
   grid_dep_launch_dependents();
@@ -369,23 +387,30 @@ __global__ void __launch_bounds__(256, 2) bank_kernel(const __grid_constant__ CU
   const uint32_t base_addr = (smem_u32(bank_smem) + 1023u) & ~1023u;  // 128-byte swizzle wants 1024-B alignment
   uint8_t *const ring = bank_smem + (base_addr - smem_u32(bank_smem));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int my_n = tiles_of_block(n_tiles);
+  const int my_n = tiles_of_block(n_tiles * sets);
   // reverse: the tiles from the end of the list, for a V larger than L2 -- the last tiles the
   // statistics pass read are still in L2 when this pass starts, and the bank tiles written last
   // (the first heads) are the first the read kernel wants
-  auto tile_of = [&](int i) {
+  auto task_of = [&](int i) {
     const int x = static_cast<int>(blockIdx.x) + i * static_cast<int>(gridDim.x);
-    return reverse ? n_tiles - 1 - x : x;
+    return reverse ? n_tiles * sets - 1 - x : x;
+  };
+  // two sets: a tile's two tasks side by side, so V comes from memory once
+  auto issue = [&](int i) {
+    const int x = task_of(i), g = sets == 2 ? x >> 1 : x;
+    bank_issue<D>(&tv, sets == 2 && (x & 1) ? bcoef1 : bcoef0, n_kt, g, base_addr + (i % kStages) * M::kSlotBytes,
+                  smem_u32(&s_full[i % kStages]));
   };
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) mbar_init(smem_u32(&s_full[s]), 1);
     fence_mbar_init();
-    for (int i = 0; i < kStages - 1 && i < my_n; ++i)
-      bank_issue<D>(&tv, bcoef, n_kt, tile_of(i), base_addr + i * M::kSlotBytes, smem_u32(&s_full[i]));
+    for (int i = 0; i < kStages - 1 && i < my_n; ++i) issue(i);
   }
   __syncthreads();
   for (int i = 0; i < my_n; ++i) {
-    const int st = i % kStages, g = tile_of(i);
+    const int st = i % kStages, x = task_of(i), g = sets == 2 ? x >> 1 : x;
+    const bool second = sets == 2 && (x & 1);
+    float *colsum = second ? colsum1 : colsum0;
     const int bh = g / n_kt, kt = g % n_kt, rows = min(kBlockK, T - kt * kBlockK);
     if (!mbar_wait(smem_u32(&s_full[st]), (i / kStages) & 1, err, kErrWaitTma)) {
       if (tid == 0) bulk_wait_group_read0();
@@ -444,16 +469,12 @@ __global__ void __launch_bounds__(256, 2) bank_kernel(const __grid_constant__ CU
     __syncthreads();
     if (tid == 0) {
 #pragma unroll
-      for (int bx = 0; bx < M::kBoxes; ++bx) tma_store_3d(&te, base_addr + st * M::kSlotBytes + bx * 16384, bx * 64,
-                                                          kt * kBlockK, bh);
+      for (int bx = 0; bx < M::kBoxes; ++bx)
+        tma_store_3d(second ? &te1 : &te0, base_addr + st * M::kSlotBytes + bx * 16384, bx * 64, kt * kBlockK, bh);
       bulk_commit_group();
       // the slot refilled next was last read by the previous tile's store
       bulk_wait_group_read<1>();
-      if (i + kStages - 1 < my_n) {
-        const int sn = (i + kStages - 1) % kStages;
-        bank_issue<D>(&tv, bcoef, n_kt, tile_of(i + kStages - 1), base_addr + sn * M::kSlotBytes,
-                      smem_u32(&s_full[sn]));
-      }
+      if (i + kStages - 1 < my_n) issue(i + kStages - 1);
     }
   }
   if (tid == 0) bulk_wait_group_read<0>();
@@ -586,7 +607,7 @@ __global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__
   // ---- plan: mode and anchor of channel grp*32 + lane, then the lazy shift walked over the tiles
   if (warp == 0) {
     const int j = grp * 32 + lane;
-    const float b = beta[h * D + j];
+    const float b = beta ? beta[h * D + j] : 0.f;
     const ChanInfo ci = chan_info(fmaxf(s_g[0][0][lane], s_g[1][0][lane]), fminf(s_g[0][1][lane], s_g[1][1][lane]),
                                   (s_g[0][2][lane] + s_g[1][2][lane]) / static_cast<float>(T), b);
     chan[bh * D + j] = ci;
@@ -692,48 +713,43 @@ __global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__
   }
 }
 
-cudaError_t launch_value_bank(const void *v, const CUtensorMap &tv, const CUtensorMap &te, const float *beta, int BH,
-                              int H, int T, int d, const BankWorkspace &w, unsigned *err, int num_sms,
-                              cudaStream_t stream, bool stats_ready) {
-  const int n_kt = (T + kBlockK - 1) / kBlockK, n_tiles = BH * n_kt;
-  const __nv_bfloat16 *vb = static_cast<const __nv_bfloat16 *>(v);
+template <int D>
+static cudaError_t launch_value_bank_d(const __nv_bfloat16 *v, const CUtensorMap &tv, const CUtensorMap &te,
+                                       const CUtensorMap *te0, const float *beta, int BH, int H, int T,
+                                       const BankWorkspace &w, const BankWorkspace *w0, unsigned *err, int num_sms,
+                                       cudaStream_t stream) {
+  const int n_kt = (T + kBlockK - 1) / kBlockK, n_tiles = BH * n_kt, sets = w0 ? 2 : 1;
   if (n_kt <= kFusedMaxTiles) {
     const size_t smem = static_cast<size_t>(n_kt) * 32 * sizeof(float);
-    if (d == 64)
-      prepass_kernel<64><<<BH * 2, 256, smem, stream>>>(vb, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
-                                                         w.colsum, w.bank);
-    else if (d == 128)
-      prepass_kernel<128><<<BH * 4, 256, smem, stream>>>(vb, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
-                                                          w.colsum, w.bank);
-    else
-      return cudaErrorInvalidValue;
+    if (w0)
+      prepass_kernel<D><<<BH * (D / 32), 256, smem, stream>>>(v, nullptr, H, T, n_kt, w0->chan, w0->shift, w0->rfac,
+                                                              w0->colmask, w0->colsum, w0->bank);
+    prepass_kernel<D><<<BH * (D / 32), 256, smem, stream>>>(v, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
+                                                            w.colsum, w.bank);
     return cudaGetLastError();
   }
-  const int grid = min(n_tiles, 2 * num_sms);
   // V larger than half of L2: the bank pass walks the tiles backwards (measured at B4 H16 T8192
   // d128: 0.7 % per step; at 25 MB, where V stays in L2, forward was 0.5 % faster)
-  const int reverse = static_cast<size_t>(n_tiles) * kBlockK * d * 2 > (size_t{64} << 20) ? 1 : 0;
-  cudaError_t e = cudaSuccess;
-  if (d == 64) {
-    using BM = BankMap<64>;
-    e = cudaFuncSetAttribute(bank_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, BM::kSmem);
-    if (e != cudaSuccess) return e;
-    if (!stats_ready) tile_stats_kernel<64><<<n_tiles, 128, 0, stream>>>(vb, T, n_kt, w.tstat);
-    plan_kernel<64><<<dim3(BH, 2), 128, 0, stream>>>(w.tstat, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
-                                                     w.bcoef);
-    bank_kernel<64><<<grid, 256, BM::kSmem, stream>>>(tv, te, w.bcoef, T, n_kt, n_tiles, reverse, w.colsum, err);
-  } else if (d == 128) {
-    using BM = BankMap<128>;
-    e = cudaFuncSetAttribute(bank_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BM::kSmem);
-    if (e != cudaSuccess) return e;
-    if (!stats_ready) tile_stats_kernel<128><<<n_tiles, 128, 0, stream>>>(vb, T, n_kt, w.tstat);
-    plan_kernel<128><<<dim3(BH, 4), 128, 0, stream>>>(w.tstat, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
-                                                      w.bcoef);
-    bank_kernel<128><<<grid, 256, BM::kSmem, stream>>>(tv, te, w.bcoef, T, n_kt, n_tiles, reverse, w.colsum, err);
-  } else {
-    return cudaErrorInvalidValue;
-  }
+  const int reverse = static_cast<size_t>(n_tiles) * kBlockK * D * 2 > (size_t{64} << 20) ? 1 : 0;
+  const BankSet a{beta, w.chan, w.shift, w.rfac, w.colmask, w.bcoef, w.colsum};
+  const BankSet b = w0 ? BankSet{nullptr, w0->chan, w0->shift, w0->rfac, w0->colmask, w0->bcoef, w0->colsum} : a;
+  using BM = BankMap<D>;
+  cudaError_t e = cudaFuncSetAttribute(bank_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, BM::kSmem);
+  if (e != cudaSuccess) return e;
+  tile_stats_kernel<D><<<n_tiles, 128, 0, stream>>>(v, T, n_kt, w.tstat);
+  plan_kernel<D><<<dim3(BH, D / 32, sets), 128, 0, stream>>>(w.tstat, a, b, H, T, n_kt);
+  bank_kernel<D><<<min(n_tiles * sets, 2 * num_sms), 256, BM::kSmem, stream>>>(
+      tv, te, w0 ? *te0 : te, a.bcoef, b.bcoef, sets, T, n_kt, n_tiles, reverse, a.colsum, b.colsum, err);
   return cudaGetLastError();
+}
+
+cudaError_t launch_value_bank(const void *v, const CUtensorMap &tv, const CUtensorMap &te, const CUtensorMap *te0,
+                              const float *beta, int BH, int H, int T, int d, const BankWorkspace &w,
+                              const BankWorkspace *w0, unsigned *err, int num_sms, cudaStream_t stream) {
+  const __nv_bfloat16 *vb = static_cast<const __nv_bfloat16 *>(v);
+  if (d == 64) return launch_value_bank_d<64>(vb, tv, te, te0, beta, BH, H, T, w, w0, err, num_sms, stream);
+  if (d == 128) return launch_value_bank_d<128>(vb, tv, te, te0, beta, BH, H, T, w, w0, err, num_sms, stream);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace fem

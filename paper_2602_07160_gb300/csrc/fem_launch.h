@@ -62,11 +62,11 @@ inline size_t fixup_capacity(size_t BH, size_t T) {
 // BankCoef, one float4 per (b, h, key tile, channel), written by the plan:
 //   linear bank   {1/beta (0 at beta = 0), beta, c_lin, NaN}
 //   shifted bank  {beta log2 e, (kBankOffset - beta c) log2 e, c, 0}
-// stats_ready: w.tstat already holds the tiles' statistics of this V (they do
-// not depend on beta); skip recomputing them.
-cudaError_t launch_value_bank(const void *v, const CUtensorMap &tv, const CUtensorMap &te, const float *beta, int BH,
-                              int H, int T, int d, const BankWorkspace &w, unsigned *err, int num_sms,
-                              cudaStream_t stream, bool stats_ready = false);
+// With te0 and w0 both given (the gated read) also the mean's plan and bank, those
+// of beta = 0, into w0; the statistics do not depend on beta and are taken once.
+cudaError_t launch_value_bank(const void *v, const CUtensorMap &tv, const CUtensorMap &te, const CUtensorMap *te0,
+                              const float *beta, int BH, int H, int T, int d, const BankWorkspace &w,
+                              const BankWorkspace *w0, unsigned *err, int num_sms, cudaStream_t stream);
 
 // Gates of the one-pass two-level gated read: o = g (mu + lambda (F - mu))
 // with mu the mean read (its bank v - c_lin, anchors chan0, column sums
