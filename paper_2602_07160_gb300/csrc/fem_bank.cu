@@ -486,18 +486,20 @@ __global__ void __launch_bounds__(256, 2) bank_kernel(const __grid_constant__ CU
 // bytes set the pre-pass's time.  One 256-thread block per (b, h) and group of
 // 32 channels: the statistics of every key tile (the tiles' maxima kept in
 // shared memory), the plan of its 32 channels, then the bank and its column
-// sums, the tiles taken from the last (the most recently read first).  Warp w
-// takes the 16-byte chunk w % 4 (channels 8 (w % 4) .. + 7 of the group) of the
-// key tiles w / 4, w / 4 + 2, ...; lane l rows l, l + 32, l + 64, l + 96 of a
-// tile, so a channel's bank form is uniform across the warp and all eight warps
-// work on sequences of two key tiles.  A warp load touches 32 row segments,
+// sums.  Warp w takes the 16-byte chunk w % 4 (channels 8 (w % 4) .. + 7 of the
+// group) of the key tiles w / 4 and, with more than two (TP = 2), w / 4 + 2; its
+// rows stay in registers from the statistics to the bank, so V is read once, and
+// those of one or two tiles leave room for four or three blocks per SM (with the rows of four
+// tiles at a time, V read again for the bank and two blocks per SM, a call at B64 H6 T197 d64 took 47.5 us
+// and takes 43.2; B32 H8 T256 d128 162 -> 152, B64 H16 T512 d128 841 -> 810).
+// Lane l takes rows l, l + 32, l + 64, l + 96 of a tile, so a channel's bank
+// form is uniform across the warp and all eight warps work on sequences of two
+// key tiles.  A warp load touches 32 row segments,
 // which costs more than the launches saved from 16 key tiles on; there the
 // three kernels run.  The results are those of the three kernels up to the
 // summation order of the channel means.
 // ---------------------------------------------------------------------------
 constexpr int kFusedMaxTiles = 4;
-constexpr int kFusedStatsTiles = 4;  // key tiles whose loads a warp keeps in flight (statistics)
-constexpr int kFusedBankTiles = 2;   // the same for the bank
 
 // Max (OP 0), min (1) or sum (2) of x[u] over the warp's 32 lanes for u = 0..7,
 // transposed like warp_sum8_transposed: lane l ends with the result for
@@ -526,8 +528,8 @@ __device__ __forceinline__ float warp_reduce8_transposed(const float (&x)[8], in
   return c;
 }
 
-template <int D>
-__global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__restrict__ v,
+template <int D, int TP>
+__global__ void __launch_bounds__(256, TP == 1 ? 4 : 3) prepass_kernel(const __nv_bfloat16 *__restrict__ v,
                                                           const float *__restrict__ beta, int H, int T, int n_kt,
                                                           ChanInfo *__restrict__ chan, float *__restrict__ shift,
                                                           float *__restrict__ rfac, unsigned *__restrict__ colmask,
@@ -549,22 +551,21 @@ __global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__
 
   // ---- statistics: max, min and sum of every tile's valid keys
   float gmx = -INFINITY, gmn = INFINITY, gsm = 0.f;  // channel j0 + ul over this warp's tiles
-  for (int kb = ph; kb < n_kt; kb += 2 * kFusedStatsTiles) {
-    uint4 raw[kFusedStatsTiles][4];
+  uint4 raw[TP][4];  // rows lane, lane + 32, ... of tiles ph, ph + 2: for the statistics, then for the bank
 #pragma unroll
-    for (int i = 0; i < kFusedStatsTiles; ++i) {
-      const int kt = kb + 2 * i;
+  for (int i = 0; i < TP; ++i) {
+    const int kt = ph + 2 * i;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = kt * kBlockK + r * 32 + lane;
-        raw[i][r] = kt < n_kt && row < T ? __ldg(reinterpret_cast<const uint4 *>(vb + static_cast<size_t>(row) * D))
-                                         : make_uint4(0u, 0u, 0u, 0u);
-      }
+    for (int r = 0; r < 4; ++r) {
+      const int row = kt * kBlockK + r * 32 + lane;
+      raw[i][r] = kt < n_kt && row < T ? __ldg(reinterpret_cast<const uint4 *>(vb + static_cast<size_t>(row) * D))
+                                       : make_uint4(0u, 0u, 0u, 0u);
     }
+  }
 #pragma unroll
-    for (int i = 0; i < kFusedStatsTiles; ++i) {
-      const int kt = kb + 2 * i;
-      if (kt >= n_kt) break;
+  for (int i = 0; i < TP; ++i) {
+    const int kt = ph + 2 * i;
+    if (kt < n_kt) {
       float mx[8], mn[8], sm[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -645,7 +646,7 @@ __global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__
     }
   }
 
-  // ---- bank: tiles from the last, E = bank(v) in fp16 and the column sums of |E|
+  // ---- bank: E = bank(v) in fp16 and the column sums of |E|
   bool lin_u[8];
   float b_u[8], cl_u[8];
 #pragma unroll
@@ -655,24 +656,10 @@ __global__ void __launch_bounds__(256, 2) prepass_kernel(const __nv_bfloat16 *__
     cl_u[u] = s_clin[8 * cq + u];
   }
   __half *eb = bank + head * D + j0;
-  const int n_mine = n_kt > ph ? (n_kt - 1 - ph) / 2 + 1 : 0;  // tiles n_kt - 1 - ph - 2 i
-  for (int i0 = 0; i0 < n_mine; i0 += kFusedBankTiles) {
-    uint4 raw[kFusedBankTiles][4];
 #pragma unroll
-    for (int i = 0; i < kFusedBankTiles; ++i) {
-      const int kt = n_kt - 1 - ph - 2 * (i0 + i);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = kt * kBlockK + r * 32 + lane;
-        raw[i][r] = i0 + i < n_mine && row < T
-                        ? __ldg(reinterpret_cast<const uint4 *>(vb + static_cast<size_t>(row) * D))
-                        : make_uint4(0u, 0u, 0u, 0u);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < kFusedBankTiles; ++i) {
-      if (i0 + i >= n_mine) break;
-      const int kt = n_kt - 1 - ph - 2 * (i0 + i);
+  for (int i = 0; i < TP; ++i) {
+    const int kt = ph + 2 * i;
+    if (kt < n_kt) {
       float res[4][8], csum[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -721,11 +708,11 @@ static cudaError_t launch_value_bank_d(const __nv_bfloat16 *v, const CUtensorMap
   const int n_kt = (T + kBlockK - 1) / kBlockK, n_tiles = BH * n_kt, sets = w0 ? 2 : 1;
   if (n_kt <= kFusedMaxTiles) {
     const size_t smem = static_cast<size_t>(n_kt) * 32 * sizeof(float);
+    const auto kern = n_kt <= 2 ? prepass_kernel<D, 1> : prepass_kernel<D, 2>;
     if (w0)
-      prepass_kernel<D><<<BH * (D / 32), 256, smem, stream>>>(v, nullptr, H, T, n_kt, w0->chan, w0->shift, w0->rfac,
-                                                              w0->colmask, w0->colsum, w0->bank);
-    prepass_kernel<D><<<BH * (D / 32), 256, smem, stream>>>(v, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask,
-                                                            w.colsum, w.bank);
+      kern<<<BH * (D / 32), 256, smem, stream>>>(v, nullptr, H, T, n_kt, w0->chan, w0->shift, w0->rfac, w0->colmask,
+                                                 w0->colsum, w0->bank);
+    kern<<<BH * (D / 32), 256, smem, stream>>>(v, beta, H, T, n_kt, w.chan, w.shift, w.rfac, w.colmask, w.colsum, w.bank);
     return cudaGetLastError();
   }
   // V larger than half of L2: the bank pass walks the tiles backwards (measured at B4 H16 T8192
