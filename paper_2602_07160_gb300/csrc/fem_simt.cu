@@ -224,6 +224,104 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
   if (lse && lane == 0) lse[row] = m + logf(L);
 }
 
+// Few rows of few keys: a block per row with every visible key in shared memory, so that nothing is
+// folded in turn.  Thread = key for the scores (K padded by one float a row: no bank conflicts), then
+// thread = channel j and key group g (C channels, 128 / C groups): the channel's largest value, then
+// sums at it over the group's keys, the groups combined through shared memory.
+//   L = sum_i P_i,  A_j = sum_i P_i exp(beta_j (v_ij - c_j)),  X_j = sum_i P_i expm1(beta_j (v_ij - c_j))
+// (X of the plain differences at beta = 0), read as above with X = beta W.  What bounds it is latency: one
+// round of loads, two block reductions and a group's exponentials.  us in a graph, four warps folding key
+// after key / this: B1 H1 T64 d16 12.5 / 4.9, B1 H1 T40 d128 26.9 / 9.4, B4 H8 T47 d64 32.1 / 14.3, B16 H4
+// T30 d128 49.7 / 21.0, B1 H1 T5 d16 3.8 / 3.2.
+constexpr int kRowThreads = 128, kRowMaxKeys = 128;
+constexpr size_t kRowSmem = 48 * 1024 - 4096;  // beside the static arrays, without an opt-in
+
+__host__ __device__ inline size_t row_floats(int T, int d) { return static_cast<size_t>(T) * (2 * d + 1) + d; }
+
+template <typename In>
+__global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restrict__ q, const In *__restrict__ k,
+                                                               const In *__restrict__ v,
+                                                               const float *__restrict__ beta, float *__restrict__ out,
+                                                               float *__restrict__ lse, int H, int T, int d, int C,
+                                                               int causal) {
+  extern __shared__ float simt_smem[];
+  __shared__ float s_p[kRowMaxKeys], s_red[2][4], s_g[3][kRowThreads];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long row = blockIdx.x, bh = row / T;
+  const int t = static_cast<int>(row % T), n = causal ? t + 1 : T, ldk = d + 1;
+  float *sk = simt_smem, *sv = sk + n * ldk, *sq = sv + n * d;
+  const In *kb = k + bh * T * d, *vb = v + bh * T * d;
+  for (int e = tid; e < n * d; e += kRowThreads) {
+    const int i = e / d;
+    sk[e + i] = ld_in(kb + e);
+    sv[e] = ld_in(vb + e);
+  }
+  for (int e = tid; e < d; e += kRowThreads) sq[e] = ld_in(q + row * d + e);
+  __syncthreads();
+  // ---- scores, their maximum, P and its sum
+  float s = -INFINITY;
+  if (tid < n) {
+    const float *kr = sk + tid * ldk;
+    float s0 = 0.f, s1 = 0.f;
+    int e = 0;
+#pragma unroll 4
+    for (; e + 1 < d; e += 2) {
+      s0 = fmaf(sq[e], kr[e], s0);
+      s1 = fmaf(sq[e + 1], kr[e + 1], s1);
+    }
+    if (e < d) s0 = fmaf(sq[e], kr[e], s0);
+    s = (s0 + s1) * rsqrtf(static_cast<float>(d));
+  }
+  float m = s;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+  if (lane == 0) s_red[0][warp] = m;
+  __syncthreads();
+  m = fmaxf(fmaxf(s_red[0][0], s_red[0][1]), fmaxf(s_red[0][2], s_red[0][3]));
+  float p = tid < n ? expf(s - m) : 0.f;
+  s_p[tid] = p;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
+  if (lane == 0) s_red[1][warp] = p;
+  // ---- channels, C at a time
+  const int G = kRowThreads / C, jl = tid % C, g = tid / C, h = static_cast<int>(bh % H);
+  for (int j0 = 0; j0 < d; j0 += C) {
+    const int j = j0 + jl;
+    const bool on = j < d;
+    const float b = on ? beta[static_cast<size_t>(h) * d + j] : 0.f;
+    float c = -INFINITY;
+    if (on) {
+#pragma unroll 4
+      for (int i = g; i < n; i += G) c = fmaxf(c, sv[i * d + j]);
+    }
+    s_g[0][tid] = c;
+    __syncthreads();  // also: P and its partial sums
+    for (int u = 0; u < G; ++u) c = fmaxf(c, s_g[0][u * C + jl]);
+    float A = 0.f, X = 0.f;
+    if (on) {
+#pragma unroll 4
+      for (int i = g; i < n; i += G) {
+        const float x = sv[i * d + j] - c, y = b * x, pi = s_p[i];
+        A = fmaf(pi, expf(y), A);
+        X = fmaf(pi, b != 0.f ? expm1f(y) : x, X);
+      }
+    }
+    s_g[1][tid] = A;
+    s_g[2][tid] = X;
+    __syncthreads();
+    const float L = (s_red[1][0] + s_red[1][1]) + (s_red[1][2] + s_red[1][3]);
+    if (g == 0 && on) {
+      for (int u = 1; u < G; ++u) {
+        A += s_g[1][u * C + jl];
+        X += s_g[2][u * C + jl];
+      }
+      const float z = X / L;
+      out[row * d + j] = b == 0.f ? c + z : z > -0.5f ? c + log1pf(z) / b : c + logf(A / L) / b;
+    }
+    if (j0 == 0 && tid == 0 && lse) lse[row] = m + logf(L);
+  }
+}
+
 template <typename In>
 static cudaError_t launch_simt(const In *q, const In *k, const In *v, const float *beta, float *out, float *lse, int B,
                                int H, int T, int d, int causal, cudaStream_t stream) {
@@ -232,6 +330,13 @@ static cudaError_t launch_simt(const In *q, const In *k, const In *v, const floa
   // states fits in the staging space: 3 (2 + 3 d) <= 2 tile d floats)
   const long long rows = static_cast<long long>(B) * H * T;
   const bool split = rows <= kSimtSplitRows;
+  if (split && T <= kRowMaxKeys && row_floats(T, d) * sizeof(float) <= kRowSmem) {
+    int C = 16;
+    while (C < d && C < kRowThreads) C *= 2;
+    fem_row_kernel<In><<<static_cast<unsigned>(rows), kRowThreads, row_floats(T, d) * sizeof(float), stream>>>(
+        q, k, v, beta, out, lse, H, T, d, C, causal);
+    return cudaGetLastError();
+  }
   const unsigned blocks = static_cast<unsigned>(split ? rows : static_cast<long long>(B) * H * ((T + 3) / 4));
   const size_t smem = 2 * static_cast<size_t>(fem_simt_tile(d)) * d * sizeof(float);
   const int per = (d + 31) / 32;
