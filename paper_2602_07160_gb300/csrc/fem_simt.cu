@@ -1,10 +1,11 @@
 // The FEM read on CUDA cores, exact to fp32 rounding: fp32 inputs of any head
 // dimension up to 256, and bf16 inputs of head dimension 16 or 32 (too narrow
 // for the tensor-core read's 64-channel tiles to pay; here every product and
-// sum is fp32).  This kernel runs the shortest sequences and d > 128, the
-// tiles of fem_f32_tile.cu the others (use_tile below).
+// sum is fp32).  fem_row_kernel runs few short rows, the tiles of
+// fem_f32_tile.cu longer sequences (use_tile below), fem_simt_kernel the rest:
+// many short rows, and d > 128.
 //
-// One warp per output row t, four consecutive rows of one (b, h) per block;
+// fem_simt_kernel: one warp per output row t, four consecutive rows of one (b, h) per block;
 // lane l owns channels l, l+32, ...  The block stages the keys' K and V rows
 // in shared memory, a tile of fem_simt_tile(d) keys at a time (as fp32), so the
 // walk below reads them with shared-memory latency.  For every key
@@ -238,6 +239,10 @@ constexpr size_t kRowSmem = 48 * 1024 - 4096;  // beside the static arrays, with
 
 __host__ __device__ inline size_t row_floats(int T, int d) { return static_cast<size_t>(T) * (2 * d + 1) + d; }
 
+static bool row_fits(long long rows, int T, int d) {
+  return rows <= kSimtSplitRows && T <= kRowMaxKeys && row_floats(T, d) * sizeof(float) <= kRowSmem;
+}
+
 template <typename In>
 __global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restrict__ q, const In *__restrict__ k,
                                                                const In *__restrict__ v,
@@ -330,7 +335,7 @@ static cudaError_t launch_simt(const In *q, const In *k, const In *v, const floa
   // states fits in the staging space: 3 (2 + 3 d) <= 2 tile d floats)
   const long long rows = static_cast<long long>(B) * H * T;
   const bool split = rows <= kSimtSplitRows;
-  if (split && T <= kRowMaxKeys && row_floats(T, d) * sizeof(float) <= kRowSmem) {
+  if (row_fits(rows, T, d)) {
     int C = 16;
     while (C < d && C < kRowThreads) C *= 2;
     fem_row_kernel<In><<<static_cast<unsigned>(rows), kRowThreads, row_floats(T, d) * sizeof(float), stream>>>(
@@ -362,7 +367,15 @@ static cudaError_t launch_simt(const In *q, const In *k, const In *v, const floa
 // B*H = 16, d = 128: T 64 58.7 / 34.8; B*H = 64, d = 16: T 16 8.5 / 11, T 32 16.9 / 12; B*H = 384,
 // d = 64: T 8 14.6 / 36, T 32 103 / 37; B*H = 4, d = 64, T 2048: 2468 / 174.  bf16, B*H = 16, d = 32,
 // T 1024: 1271 / 56.
+// Before it, fem_row_kernel while all rows' keys and channels (the whole square) are 4 M at most: that
+// kernel / the tiled one, us in a graph: B*H = 1 T 80 d 16 4.7 / 13.5, T 80 d 64 9.0 / 18.4; B*H = 4 T 128
+// d 16 6.7 / 14.0; B*H = 8 T 100 d 32 10.1 / 12.7; B*H = 16 T 128 d 16 (4.2 M) 13.9 / 13.9; beyond, B*H = 32
+// T 64 d 64 21.9 / 17.3, B*H = 16 T 128 d 32 21.3 / 12.9.
+constexpr long long kRowWork = 1ll << 22;
+
 static bool use_tile(int B, int H, int T, int d, int max_d) {
+  const long long rows = static_cast<long long>(B) * H * T;
+  if (row_fits(rows, T, d) && rows * T * d <= kRowWork) return false;
   const bool long_enough = T >= 80 || (T >= 48 && d > 32) || (T >= 32 && static_cast<long long>(B) * H >= 64);
   return d <= max_d && long_enough && T <= kTileMaxT;
 }

@@ -23,7 +23,8 @@ def lib():
 @pytest.mark.parametrize("B,H,T,d,causal,scale", [(1, 1, 1, 16, True, 1.0), (1, 1, 64, 16, True, 1.0), (2, 3, 79, 32, False, 1.0),
                                                   (1, 2, 33, 1, True, 1.0), (1, 2, 47, 17, False, 1.0), (1, 2, 40, 128, True, 1.0),
                                                   (1, 2, 47, 128, True, 1.0), (1, 1, 20, 256, False, 1.0), (1, 2, 31, 130, True, 1.0),
-                                                  (1, 2, 64, 16, True, 8.0)])
+                                                  (1, 2, 64, 16, True, 8.0), (1, 1, 128, 16, True, 1.0), (1, 8, 100, 32, True, 1.0),
+                                                  (1, 1, 87, 64, False, 1.0)])
 def test_short_rows(B, H, T, d, causal, scale, dtype):
     if dtype == "bf16" and d not in (16, 32):
         pytest.skip("the bf16 read takes d 16 and 32 here")
