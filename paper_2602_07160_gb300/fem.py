@@ -91,8 +91,8 @@ def load(path: str | None = None):
 # interpreter steps: addresses go to the ABI as plain integers, the current stream's handle comes
 # without a Stream object, and each group of checks is one expression whose failure goes through the
 # tensors one by one for the message.  Per call without the C function: fem_fwd_f32 13.2 -> 6.0 us,
-# fem_decode 12.2 -> 5.6, fem_tdc_conv 7.5 -> 2.9 (B1 H1 T64 d16 then takes 14.3 us a call, the kernel's own
-# time, instead of 21.6).
+# fem_decode 12.2 -> 5.6, fem_tdc_conv 7.5 -> 2.9 (an fp32 call at B1 H1 T64 d16 went from 21.6 to
+# 14.3 us with it, the kernel's time then).
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
