@@ -16,6 +16,11 @@
 // A channel is linear when beta times the spread of v is at most 4 (c the mean,
 // clamped so that a lies in [-1, 3]): no difference of large terms.  The shifted
 // channels' c is the middle of the spread, so e^a and e^b stay within e^+-kWideExp.
+// The cotangents enter Z and R over a power of two of their row (its largest, g' in
+// [1, 2) there), which comes back at dS; the sums over rows take p times the row's
+// power over the head's largest, which comes back at dv and dbeta.  So nothing depends
+// on the scale of g, and what fp32's range drops from p e^b (2^-150) stays, times e^a,
+// below 2^-46 of the head's largest cotangent.
 // All exponents carry their rounding errors (exp_tilt), which keeps the gradients'
 // error at that of exp(x) taken directly.  Channels whose spread exceeds that (or is
 // not finite) take no part in the contractions; their terms are formed pair by pair
@@ -41,7 +46,7 @@ namespace {
 
 constexpr int kBT = 64;           // rows and keys of a tile (rows of the other side: kRows below)
 constexpr int kBLd = 68;          // leading dimension of a transposed 64-row tile
-constexpr float kWideExp = 85.f;  // largest |a|, |b| of a factored channel
+constexpr float kWideExp = 72.f;  // largest |a|, |b| of a factored channel: 2^+-104
 constexpr float kPeakLog = -60.f;
 
 // Per (b, h, channel): {beta, 1/beta (0 at 0), c, mode}: 1 linear, 0 shifted, 2 wide.  The wide
@@ -77,8 +82,9 @@ __global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict_
     const float b = beta[(bh % H) * d + j], mean = sm / static_cast<float>(T), lo = mx - 3.f / b, hi = mn + 1.f / b;
     const bool lin = !(b > 0.f) || lo <= hi;
     const float c = lin ? (b > 0.f ? fminf(fmaxf(mean, lo), hi) : mean) : 0.5f * (mx + mn);
-    // not finite (also a sum that overflowed), or too wide for the factors
-    const bool wd = !(fabsf(sm) < INFINITY) || !(mx - mn < INFINITY) || !(0.5f * b * (mx - mn) <= kWideExp);
+    // not finite (also a sum that overflowed), or too wide for the factors (e^a / beta among them)
+    const bool wd = !(fabsf(sm) < INFINITY) || !(mx - mn < INFINITY) ||
+                    !(lin || 0.5f * b * (mx - mn) + fmaxf(-logf(b), 0.f) <= kWideExp);
     if (wd) {
       int *list = wide + static_cast<size_t>(bh) * (d + 1);
       list[1 + atomicAdd(list, 1)] = j;
@@ -142,6 +148,12 @@ __device__ __forceinline__ float row_term(const Chan4 &q, int u, float o, float 
   if (q.lin[u] > 1.f) return 0.f;
   return q.lin[u] != 0.f ? g * em1_tilt(q.b[u], q.ib[u], q.c[u], o) : -g * q.ib[u];
 }
+
+// The power of two at or below m, the largest finite |g| of a row, where it and its reciprocal are normal.
+__device__ __forceinline__ float row_power(float m) {
+  return fminf(fmaxf(__int_as_float(__float_as_int(m) & 0x7f800000), 0x1p-126f), 0x1p126f);
+}
+__device__ __forceinline__ float finite_abs(float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.f; }
 
 // One wide channel's terms of a visible pair with log-weight lp, each from its own exponent:
 // q = p e^x, p expm1(x)/b and p phi(x)/b^2 with x = b (v - o).
@@ -237,7 +249,8 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
     bwd_row_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
                    const float4 *__restrict__ chan, const int *__restrict__ wide, int *__restrict__ peaked,
-                   float *__restrict__ dbp, float *__restrict__ dq, int T, int d, int causal) {
+                   float *__restrict__ power, float *__restrict__ head_power, float *__restrict__ dbp,
+                   float *__restrict__ dq, int T, int d, int causal) {
   using Lay = RowLay<DP>;
   constexpr int NC = DP / 16, CQ = DP / 4, kShare = kBT * CQ / 256;
   extern __shared__ __align__(16) float bwd_smem[];
@@ -253,10 +266,26 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
   const bool vec = (d & 3) == 0;
   const float inv_sqrt_d = rsqrtf(static_cast<float>(d));
   if (tid < DP) sDb[tid] = 0.f;
-  __syncthreads();
   {
     const int r = tid & 63, t = min(t0 + r, T - 1);
     const bool valid = t0 + r < T;
+    // the row's power of two, for the key pass as well (its partial maxima in the space of dS)
+    float gm = 0.f;
+    for (int jq = tid >> 6; jq < CQ; jq += 4) {
+      const float4 g4 = ld_row4(dout + base + static_cast<size_t>(t) * d, jq * 4, d, vec);
+      gm = fmaxf(fmaxf(gm, fmaxf(finite_abs(g4.x), finite_abs(g4.y))), fmaxf(finite_abs(g4.z), finite_abs(g4.w)));
+    }
+    sS[tid] = gm;
+    __syncthreads();
+    const float pw = row_power(fmaxf(fmaxf(sS[r], sS[kBT + r]), fmaxf(sS[2 * kBT + r], sS[3 * kBT + r]))), ipw = 1.f / pw;
+    if (tid < kBT) {
+      sS[4 * kBT + r] = pw;
+      if (rank == 0 && valid) {
+        power[static_cast<size_t>(bh) * T + t] = pw;
+        // positive floats order as their bits
+        atomicMax(reinterpret_cast<int *>(head_power) + bh, __float_as_int(pw));
+      }
+    }
     float R = 0.f;
     for (int jq = tid >> 6; jq < CQ; jq += 4) {
       const int j = jq * 4;
@@ -269,8 +298,8 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float g = valid ? gv[u] : 0.f;
-        z[u] = row_factor(cp, u, ov[u], g);
-        R += row_term(cp, u, ov[u], g);
+        z[u] = row_factor(cp, u, ov[u], g * ipw);
+        R += row_term(cp, u, ov[u], g * ipw);
         db[u] = cp.lin[u] > 1.f ? 0.f
                                 : (cp.lin[u] != 0.f ? g * phi_over_b2(cp.b[u], cp.ib[u], cp.c[u], ov[u]) : g * cp.ib[u] * cp.ib[u]);
       }
@@ -290,10 +319,11 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
   }
   __syncthreads();
   if (rank == 0 && tid < d) atomicAdd(dbp + static_cast<size_t>(bh) * d + tid, sDb[tid]);
-  float R[4], ls[4];
+  float R[4], ls[4], pw[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int row = ty * 4 + r;
+    pw[r] = sS[4 * kBT + row];
     R[r] = (sR[row] + sR[kBT + row]) + (sR[2 * kBT + row] + sR[3 * kBT + row]);
     ls[r] = lse[static_cast<size_t>(bh) * T + min(t0 + row, T - 1)];
   }
@@ -349,7 +379,7 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
         const float l = fmaf(sv, inv_sqrt_d, -ls[r]);
         peak = peak || (vis && l < kPeakLog);
         lp[c][r] = vis ? l : -INFINITY;
-        ds[c][r] = vis ? expf(l) * (uv + R[r]) : 0.f;
+        ds[c][r] = vis ? expf(l) * (uv + R[r]) * pw[r] : 0.f;
       }
     }
     for (int w = 0; w < n_wide; ++w) {
@@ -425,7 +455,8 @@ __global__ void __launch_bounds__(256, 1)
     bwd_key_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
                    const float4 *__restrict__ chan, const int *__restrict__ wide, int *__restrict__ peaked,
-                   float *__restrict__ dbp, float *__restrict__ dk, float *__restrict__ dv, int T, int d, int causal) {
+                   const float *__restrict__ power, const float *__restrict__ head_power, float *__restrict__ dbp,
+                   float *__restrict__ dk, float *__restrict__ dv, int T, int d, int causal) {
   using Lay = KeyLay<DP>;
   constexpr int NC = DP / 16, CQ = DP / 4, kRows = Lay::kRows, RR = Lay::RR, kRl = Lay::kRl, kNl = Lay::kNl;
   extern __shared__ __align__(16) float bwd_smem[];
@@ -439,7 +470,7 @@ __global__ void __launch_bounds__(256, 1)
   const size_t base = static_cast<size_t>(bh) * T * d;
   const float4 *ch = chan + static_cast<size_t>(bh) * d;
   const bool vec = (d & 3) == 0;
-  const float inv_sqrt_d = rsqrtf(static_cast<float>(d));
+  const float inv_sqrt_d = rsqrtf(static_cast<float>(d)), hpw = head_power[bh], ihpw = 1.f / hpw;
   if (tid < DP) sDb[tid] = 0.f;
   for (int e = tid; e < kBT * CQ; e += 256) {
     const int r = e & 63, j = (e >> 6) * 4;
@@ -466,6 +497,7 @@ __global__ void __launch_bounds__(256, 1)
     {
       const int r = tid % kRows, t = min(t0 + r, T - 1);
       const bool valid = t0 + r < T;
+      const float ipw = 1.f / power[static_cast<size_t>(bh) * T + t];
       float R = 0.f;
       for (int jq = tid / kRows; jq < CQ; jq += Lay::kParts) {
         const int j = jq * 4;
@@ -477,7 +509,7 @@ __global__ void __launch_bounds__(256, 1)
         float z[4], z2[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const float g = valid ? gv[u] : 0.f;
+          const float g = valid ? gv[u] * ipw : 0.f;
           z[u] = row_factor(cp, u, ov[u], g);
           z2[u] = cp.lin[u] > 1.f ? 0.f : z[u] * (cp.c[u] - ov[u]);
           R += row_term(cp, u, ov[u], g);
@@ -517,7 +549,8 @@ __global__ void __launch_bounds__(256, 1)
       float Rt = 0.f;
 #pragma unroll
       for (int p = 0; p < Lay::kParts; ++p) Rt += sR[p * kRows + row];
-      const float ls = lse[static_cast<size_t>(bh) * T + min(t, T - 1)];
+      const float ls = lse[static_cast<size_t>(bh) * T + min(t, T - 1)], pw = power[static_cast<size_t>(bh) * T + min(t, T - 1)];
+      const float prel = pw * ihpw;
       float pv[4];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -528,9 +561,10 @@ __global__ void __launch_bounds__(256, 1)
         peak = peak || (vis && l < kPeakLog);
         lp[r][c] = vis ? l : -INFINITY;
         pv[c] = vis ? expf(l) : 0.f;
-        ds[r][c] = vis ? pv[c] * (uv + Rt) : 0.f;
+        ds[r][c] = vis ? pv[c] * (uv + Rt) * pw : 0.f;
       }
-      *reinterpret_cast<float4 *>(sP + row * kBT + tx * 4) = make_float4(pv[0], pv[1], pv[2], pv[3]);
+      *reinterpret_cast<float4 *>(sP + row * kBT + tx * 4) =
+          make_float4(pv[0] * prel, pv[1] * prel, pv[2] * prel, pv[3] * prel);
     }
     for (int w = 0; w < n_wide; ++w) {
       const int j = wl[1 + w];
@@ -602,13 +636,13 @@ __global__ void __launch_bounds__(256, 1)
       const float vi = v[o], h = x[c * 12 + 4 + r], h2 = x[c * 12 + 8 + r], F = exp_tilt(cp.x, vi, cp.z);
       dk[o] = x[c * 12 + r] * inv_sqrt_d;
       if (cp.w > 1.f) continue;
-      dv[o] = F * h;
+      dv[o] = F * h * hpw;
       if (cp.w != 0.f)
         db += phi_over_b2(cp.x, cp.y, vi, cp.z) * h + em1_tilt(cp.x, cp.y, vi, cp.z) * h2;
       else
         db += F * fmaf(fmaf(cp.x, vi - cp.z, -1.f), h, cp.x * h2) * cp.y * cp.y;
     }
-    if (cp.w <= 1.f) atomicAdd(sDb + j, db);
+    if (cp.w <= 1.f) atomicAdd(sDb + j, db * hpw);
   }
   __syncthreads();
   if (tid < d) atomicAdd(dbp + static_cast<size_t>(bh) * d + tid, sDb[tid]);
@@ -629,17 +663,19 @@ __global__ void bwd_dbeta_kernel(const float *__restrict__ tile, const float *__
 }
 
 struct BwdWs {
-  size_t chan, tile, pairs, wide, peaked, total, zero_from;
+  size_t chan, power, tile, pairs, wide, peaked, head_power, total, zero_from;
 };
-BwdWs bwd_ws(int BH, int d) {
+BwdWs bwd_ws(int BH, int T, int d) {
   BwdWs w;
   const size_t n = static_cast<size_t>(BH) * d;
   w.chan = 0;
-  w.zero_from = w.tile = n * sizeof(float4);
+  w.power = n * sizeof(float4);  // the rows' powers of two
+  w.zero_from = w.tile = w.power + static_cast<size_t>(BH) * T * sizeof(float);
   w.pairs = w.tile + n * sizeof(float);
   w.wide = w.pairs + n * sizeof(float);
   w.peaked = w.wide + (n + BH) * sizeof(int);
-  w.total = w.peaked + static_cast<size_t>(BH) * sizeof(int);
+  w.head_power = w.peaked + static_cast<size_t>(BH) * sizeof(int);
+  w.total = w.head_power + static_cast<size_t>(BH) * sizeof(float);
   return w;
 }
 
@@ -667,7 +703,8 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
                            const float *lse, const float *dout, float *dq, float *dk, float *dv, int BH, int H, int T,
                            int d, int causal, uint8_t *ws, const BwdWs &w, int num_sms, cudaStream_t stream) {
   float4 *chan = reinterpret_cast<float4 *>(ws + w.chan);
-  float *tile = reinterpret_cast<float *>(ws + w.tile);
+  float *tile = reinterpret_cast<float *>(ws + w.tile), *power = reinterpret_cast<float *>(ws + w.power),
+        *head_power = reinterpret_cast<float *>(ws + w.head_power);
   int *wide = reinterpret_cast<int *>(ws + w.wide), *peaked = reinterpret_cast<int *>(ws + w.peaked);
   const int n_t = (T + kBT - 1) / kBT;
   bwd_chan_kernel<<<dim3(BH, (d + 31) / 32), 1024, 0, stream>>>(v, beta, H, T, d, chan, wide, dv);
@@ -677,11 +714,12 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = launch_cluster(bwd_row_kernel<DP>, dim3(size, n_t, BH), RowLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
-                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, tile, dq, T, d, causal);
+                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, power, head_power, tile, dq, T, d,
+                       causal);
   if (e == cudaSuccess)
     e = launch_cluster(bwd_key_kernel<DP>, dim3(size, n_t, BH), KeyLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
-                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, tile, dk, dv, T, d,
-                       causal);
+                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, static_cast<const float *>(power),
+                       static_cast<const float *>(head_power), tile, dk, dv, T, d, causal);
   return e;
 }
 
@@ -695,7 +733,7 @@ bool bwd_tile_takes(int B, int H, int T, int d) {
 }
 
 size_t bwd_workspace_bytes(int B, int H, int T, int d) {
-  return bwd_tile_takes(B, H, T, d) ? bwd_ws(B * H, d).total : 0;
+  return bwd_tile_takes(B, H, T, d) ? bwd_ws(B * H, T, d).total : 0;
 }
 
 cudaError_t launch_bwd_tile(const float *q, const float *k, const float *v, const float *beta, const float *out,
@@ -703,7 +741,7 @@ cudaError_t launch_bwd_tile(const float *q, const float *k, const float *v, cons
                             int H, int T, int d, int causal, void *ws, int num_sms, cudaStream_t stream) {
   const int BH = B * H;
   uint8_t *p = static_cast<uint8_t *>(ws);
-  const BwdWs w = bwd_ws(BH, d);
+  const BwdWs w = bwd_ws(BH, T, d);
   cudaError_t e = cudaMemsetAsync(p + w.zero_from, 0, w.total - w.zero_from, stream);
   if (e != cudaSuccess) return e;
   if (d <= 32)
