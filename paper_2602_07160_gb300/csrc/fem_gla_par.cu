@@ -651,8 +651,10 @@ __global__ void __launch_bounds__(256, 2) gla_out_kernel(const float *__restrict
           const float sum = dl >= 0.f ? fmaf(ix, ed, in) : fmaf(in, ed, ix);
           flag |= !(in >= zmin) ? 1u << (q * 8 + u) : 0u;
           o[u] = ((fmaxf(pj.z, lb) - lz2) + lg2_approx(sum)) * pj.y;
-          if (!(sum > 0x1p-100f) && in > 0.f) {  // the larger scale's part too small to be the shift
-            const float la2 = pj.z + lg2_approx(in), lb2 = ix > 0.f ? lb + lg2_approx(ix) : -INFINITY;
+          // the larger scale's part too small to be the shift (or none, for features that meet no key of the chunk)
+          if (!(sum > 0x1p-100f) && (in > 0.f || ix > 0.f)) {
+            const float la2 = in > 0.f ? pj.z + lg2_approx(in) : -INFINITY,
+                        lb2 = ix > 0.f ? lb + lg2_approx(ix) : -INFINITY;
             o[u] = ((fmaxf(la2, lb2) - lz2) + lg2_approx(1.f + ex2_approx(-fabsf(la2 - lb2)))) * pj.y;
           }
         }
