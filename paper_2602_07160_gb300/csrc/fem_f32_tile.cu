@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
         gn = fminf(gn, r[2]);
         gs += r[3];
       }
-      const float b = j < d ? beta[h * d + j] : 0.f, mean = gs / static_cast<float>(n_keys);
+      const float b = j < d ? normal_beta(beta[h * d + j]) : 0.f, mean = gs / static_cast<float>(n_keys);
       bool lin = true;
       float c = mean;
       if (b > 0.f) {

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(128) gla_stats_kernel(const float *__restrict_
 __global__ void __launch_bounds__(256) gla_anchor_kernel(const float *__restrict__ beta, int h0, int H, int T, int n_ch,
                                                          GlaTcWs w) {
   const int lane = threadIdx.x & 31, j = blockIdx.x * 8 + (threadIdx.x >> 5), hd = blockIdx.y;
-  const float b = beta[((h0 + hd) % H) * kGD + j];
+  const float b = normal_beta(beta[((h0 + hd) % H) * kGD + j]);
   const bool shifted = b >= kGlaLinBeta;
   const size_t t0 = static_cast<size_t>(hd) * n_ch;
   float rmin = INFINITY, rsum = 0.f, c_old = INFINITY, mu = -INFINITY;  // carried over the groups of 32 chunks
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(256, 3) gla_local_kernel(const float *__restri
   __syncthreads();
   {
     // the bank: 8 keys' entries to a 16-byte chunk
-    const float b = beta[((h0 + hd) % H) * kGD + j], sh = w.shift[task * kGD + j], rb = b != 0.f ? 1.f / b : 0.f;
+    const float b = normal_beta(beta[((h0 + hd) % H) * kGD + j]), sh = w.shift[task * kGD + j], rb = b != 0.f ? 1.f / b : 0.f;
     const bool lin = b < kGlaLinBeta;
 #pragma unroll
     for (int kc = 0; kc < 4; ++kc) {
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(256, 2) gla_out_kernel(const float *__restrict
     }
     const float sz = tid < kGM ? w.s[task * kSt + kGD * kGM + tid] : 0.f;
     if (tid < kGD) {
-      const float bj = beta[((h0 + hd) % H) * kGD + tid], sh = w.shift[task * kGD + tid];
+      const float bj = normal_beta(beta[((h0 + hd) % H) * kGD + tid]), sh = w.shift[task * kGD + tid];
       par[tid] = bj >= kGlaLinBeta ? make_float4(bj, kLn2 / bj, sh * kLog2e, w.mu[task * kGD + tid] * kLog2e)
                                    : make_float4(bj, bj != 0.f ? 1.f / bj : 0.f, sh, 0.f);
     }

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(256, 1)
   for (int i = tid; i < kGN * 8; i += 256)
     *reinterpret_cast<uint4 *>(smem + GLay::kS16 + sw128_offset(i >> 3, i & 7)) = make_uint4(0u, 0u, 0u, 0u);
   for (int j = tid; j < kGN; j += 256) {
-    c_beta[j] = j < kGD ? beta[h * kVD + jo + j] : 0.f;
+    c_beta[j] = j < kGD ? normal_beta(beta[h * kVD + jo + j]) : 0.f;
     c_anc[j] = INFINITY;
     c_mu[j] = -INFINITY;
     c_lam[j] = 0.f;

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
     const int j = lane + 32 * u;
     const bool ok = valid && u < per && j < d;
     qv[u] = ok ? ld_in(q + row * d + j) : 0.f;
-    bj[u] = ok ? beta[h * d + j] : 0.f;
+    bj[u] = ok ? normal_beta(beta[h * d + j]) : 0.f;
     c[u] = -INFINITY;
     A[u] = 0.f;
     W[u] = 0.f;
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restri
   for (int j0 = 0; j0 < d; j0 += C) {
     const int j = j0 + jl;
     const bool on = j < d;
-    const float b = on ? beta[static_cast<size_t>(h) * d + j] : 0.f;
+    const float b = on ? normal_beta(beta[static_cast<size_t>(h) * d + j]) : 0.f;
     float c = -INFINITY;
     if (on) {
 #pragma unroll 4
