@@ -12,6 +12,11 @@
 // a constant channel (the paper's "constant 1 channel").  At beta_j = 0 the
 // state carries v itself and o is the ratio (the prior mean).
 //
+// So is a channel whose beta is below kGlaSmallBeta and whose values stay within kGlaSmallTilt / beta: its
+// state carries expm1(beta v) / beta and o is log1p(beta ratio) / beta, since the two logarithms' rounding
+// (some 5e-7) over beta would be 0.5 at beta = 1e-6.  Its beta goes negated through the kernels, as the
+// first launch leaves it (2.5 us where no beta is that small, under the next launch's loads).
+//
 // In chunks of 64 steps, with gamma_t the running sum of g in the chunk, three
 // launches of fp32 contractions on CUDA cores (a lone chunk needs only the last):
 //
@@ -48,6 +53,7 @@ constexpr int kThreads = 256;         // thread (ty, tx): four rows (or features
 constexpr int kLd = kSteps + 4;       // leading dimension of the transposed Q and K tiles
 constexpr float kGlaGuard = 0x1p-90f;
 constexpr float kGlaFloor = -1e6f;
+constexpr float kGlaSmallBeta = 0x1p-5f, kGlaSmallTilt = 0.25f;
 
 // Workspace of a group of heads and a run of chunks; per (head, chunk) unless noted.
 struct GlaWs {
@@ -57,6 +63,7 @@ struct GlaWs {
   float *mu;     // [dp]: the start state's
   float *gl;     // the chunk's summed log-decay
   float *carry;  // per head: [M][dp], [M] and [dp], the state (and mu) behind the run's last chunk
+  float *eb;     // per head: [dp], beta as form_beta gives it
 };
 
 // gam[t] = g_0 + ... + g_t as a float pair (steps past the end add nothing); by warp 0.
@@ -101,13 +108,68 @@ __device__ __forceinline__ float4 beta4(const float *beta, int h, int d, int j) 
   return make_float4(j < d ? p[j] : 0.f, j + 1 < d ? p[j + 1] : 0.f, j + 2 < d ? p[j + 2] : 0.f, j + 3 < d ? p[j + 3] : 0.f);
 }
 
+// beta of a channel whose largest |v| is top: 0 (the mean), negated for the small-beta form, else itself.
+__device__ __forceinline__ float form_beta(float b, float top) {
+  if (!(b >= 0x1p-126f)) return b == b ? 0.f : b;  // see normal_beta
+  return b < kGlaSmallBeta && b * top <= kGlaSmallTilt ? -b : b;
+}
+__device__ __forceinline__ bool maybe_small(float4 b) {
+  return fminf(fminf(b.x > 0.f ? b.x : 1.f, b.y > 0.f ? b.y : 1.f), fminf(b.z > 0.f ? b.z : 1.f, b.w > 0.f ? b.w : 1.f)) <
+         kGlaSmallBeta;
+}
+__device__ __forceinline__ float4 abs_max(float4 a, float4 x) {
+  return make_float4(fmaxf(a.x, fabsf(x.x)), fmaxf(a.y, fabsf(x.y)), fmaxf(a.z, fabsf(x.z)), fmaxf(a.w, fabsf(x.w)));
+}
+__device__ __forceinline__ float4 form_beta4(float4 b, float4 top) {
+  return make_float4(form_beta(b.x, top.x), form_beta(b.y, top.y), form_beta(b.z, top.z), form_beta(b.w, top.w));
+}
+
+// A value as a linear channel's state carries it: expm1(beta x) / beta for the small-beta form (x times
+// the series of expm1(y) / y, |y| <= 1/4), and the read of such a channel's ratio.
+__device__ __forceinline__ float lin_value(float b, float x) {
+  const float y = -b * x;
+  float p = fmaf(y, 1.f / 720.f, 1.f / 120.f);
+  p = fmaf(y, p, 1.f / 24.f);
+  p = fmaf(y, p, 1.f / 6.f);
+  p = fmaf(y, p, 0.5f);
+  p = fmaf(y, p, 1.f);
+  return b < 0.f ? x * p : x;
+}
+__device__ __forceinline__ void lin_values(float4 b, float4 (&x)[4]) {
+  if (b.x < 0.f || b.y < 0.f || b.z < 0.f || b.w < 0.f) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      x[u] = make_float4(lin_value(b.x, x[u].x), lin_value(b.y, x[u].y), lin_value(b.z, x[u].z), lin_value(b.w, x[u].w));
+  }
+}
+__device__ __noinline__ float small_read(float b, float ratio) { return log1pf(-b * ratio) / -b; }
+__device__ __forceinline__ float lin_read(float b, float ratio) { return b < 0.f ? small_read(b, ratio) : ratio; }
+
+// ---------------------------------------------------------------------------
+// form: block per head and 64 channels; reads the values only where some beta is small.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kThreads) gla_form_f32_kernel(const float *__restrict__ v, const float *__restrict__ beta,
+                                                                int h0, int H, int T, int d, int dp, int vec, GlaWs w) {
+  grid_dep_launch_dependents();
+  __shared__ float4 red[16][16];
+  const int tid = threadIdx.x, ty = tid >> 4, jq = blockIdx.y * kCh + (tid & 15) * 4, hd = blockIdx.x;
+  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
+  float4 top = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (__syncthreads_or(maybe_small(b))) {
+    const float *vh = v + static_cast<size_t>(h0 + hd) * T * d;
+#pragma unroll 8
+    for (int r = ty; r < T; r += 16) top = abs_max(top, ld_row4(vh + static_cast<size_t>(r) * d, jq, d, vec));
+    top = max_over_rows(top, red);
+  }
+  if (ty == 0) *reinterpret_cast<float4 *>(w.eb + static_cast<size_t>(hd) * dp + jq) = form_beta4(b, top);
+}
+
 // ---------------------------------------------------------------------------
 // local: block per chunk and 64 channels.
 // ---------------------------------------------------------------------------
 template <int M>
-__global__ void __launch_bounds__(kThreads) gla_local_f32_kernel(const float *__restrict__ kf, const float *__restrict__ v,
-                                                                 const float *__restrict__ logdecay,
-                                                                 const float *__restrict__ beta, int h0, int H, int T,
+__global__ void __launch_bounds__(kThreads, 4) gla_local_f32_kernel(const float *__restrict__ kf, const float *__restrict__ v,
+                                                                 const float *__restrict__ logdecay, int h0, int T,
                                                                  int d, int dp, int c0, int nb, int vec, GlaWs w) {
   constexpr int RT = M / 16;  // features of a thread
   __shared__ __align__(16) float sK[kSteps * M], sE[kSteps * kCh];
@@ -135,7 +197,9 @@ __global__ void __launch_bounds__(kThreads) gla_local_f32_kernel(const float *__
   if (tid < kSteps) s_dg[tid] = sum_diff(gam[kSteps - 1], gam[tid]);
   if (tid == 0 && blockIdx.y == 0) w.gl[task] = gam[kSteps - 1].x;
   __syncthreads();
-  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
+  grid_dep_wait();  // eb: a dependent launch on the form kernel, which a block's loads overlap
+  const float4 b = ld4(w.eb + static_cast<size_t>(hd) * dp + jq);
+  lin_values(b, x);
   float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   float4 y[4];
 #pragma unroll
@@ -195,8 +259,7 @@ __global__ void __launch_bounds__(kThreads) gla_local_f32_kernel(const float *__
 // chunks in turn, the start states in U's place.  Bound by the states' bytes (from L2 at moderate
 // sizes); kAhead chunks' loads in flight, the scales' chain ahead of the exponentials.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gla_scan_f32_kernel(const float *__restrict__ beta, int h0, int H, int d, int dp,
-                                                           int M, int first, int n, int nb, GlaWs w) {
+__global__ void __launch_bounds__(256) gla_scan_f32_kernel(int d, int dp, int M, int first, int n, int nb, GlaWs w) {
   constexpr int kAhead = 8;
   const int i = blockIdx.x * 256 + threadIdx.x, hd = blockIdx.y;
   if (i >= M * dp + M) return;
@@ -206,7 +269,7 @@ __global__ void __launch_bounds__(256) gla_scan_f32_kernel(const float *__restri
   const size_t t0 = static_cast<size_t>(hd) * nb, stride = is_z ? M : static_cast<size_t>(M) * dp;
   float *s = is_z ? w.z + t0 * M + (i - M * dp) : w.u + t0 * M * dp + i;
   float *carry = w.carry + static_cast<size_t>(hd) * (M * dp + M + dp);
-  const bool scaled = !is_z && beta[static_cast<size_t>((h0 + hd) % H) * d + j] > 0.f, wr_mu = !is_z && i < dp;
+  const bool scaled = !is_z && w.eb[static_cast<size_t>(hd) * dp + j] > 0.f, wr_mu = !is_z && i < dp;
   float S = first ? 0.f : carry[i], mu = !scaled ? 0.f : first ? -INFINITY : carry[M * dp + M + j];
   for (int c = 0; c < n; c += kAhead) {
     float u[kAhead], lam[kAhead], gl[kAhead], fr[kAhead], fl[kAhead], at[kAhead];
@@ -255,7 +318,8 @@ struct OutF32 {
   static constexpr int kFloats = kS + kSteps * kSteps;
 };
 
-template <int M>
+// LONE: the sequence is one chunk, so there is no state and the forms are found here.
+template <int M, bool LONE>
 __global__ void __launch_bounds__(kThreads, 3)
     gla_out_f32_kernel(const float *__restrict__ qf, const float *__restrict__ kf, const float *__restrict__ v,
                        const float *__restrict__ logdecay, const float *__restrict__ beta, float *__restrict__ out,
@@ -267,12 +331,13 @@ __global__ void __launch_bounds__(kThreads, 3)
   __shared__ float4 red[16][16];
   __shared__ float2 gam[kSteps];
   __shared__ float s_den[kSteps], s_sz[M];
+  __shared__ __align__(16) float s_b[kCh];
   __shared__ unsigned s_flag[kSteps][2];
   const int tid = threadIdx.x, lane = tid & 31, ty = tid >> 4, tx = tid & 15, hd = blockIdx.z, j0 = blockIdx.y * kCh, jq = j0 + tx * 4;
   const int c = c0 + blockIdx.x, rows = min(kSteps, T - c * kSteps);
   const size_t r0 = static_cast<size_t>(h0 + hd) * T + static_cast<size_t>(c) * kSteps;
   const size_t task = static_cast<size_t>(hd) * nb + blockIdx.x;
-  const bool state = c > 0;
+  const bool state = !LONE && c > 0;
   float4 x[4], qx[M / 16], kx[M / 16];
 #pragma unroll
   for (int u = 0; u < M / 16; ++u) {  // lanes over rows: the transposed stores hit distinct banks
@@ -307,7 +372,22 @@ __global__ void __launch_bounds__(kThreads, 3)
     sK[(f + 2) * kLd + r] = kx[u].z;
     sK[(f + 3) * kLd + r] = kx[u].w;
   }
-  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
+  float4 b;
+  if constexpr (!LONE) {
+    b = ld4(w.eb + static_cast<size_t>(hd) * dp + jq);
+  } else {
+    b = beta4(beta, (h0 + hd) % H, d, jq);
+    float4 top = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (__syncthreads_or(maybe_small(b))) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) top = abs_max(top, x[u]);
+      top = max_over_rows(top, red);
+      __syncthreads();  // red is used again
+    }
+    b = form_beta4(b, top);
+  }
+  if (ty == 0) *reinterpret_cast<float4 *>(s_b + tx * 4) = b;
+  lin_values(b, x);
   float lam[4];
   {
     float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
@@ -453,6 +533,7 @@ __global__ void __launch_bounds__(kThreads, 3)
       } else {
         flag |= !(fabsf(a) < INFINITY) ? 1u << q : 0u;
         o[q] = (state ? fmaf(et, y, a) : a) * rden;
+        if (bj[q] < 0.f) o[q] = lin_read(bj[q], o[q]);
       }
       if (jq + q >= d) flag &= ~(1u << q);
     }
@@ -500,7 +581,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     __syncwarp();
     // the read from the in-chunk sum acc at the shift m (linear: acc alone) and the state's part
     auto read = [&](float bq, float m, float acc, float ixe, int j) {
-      if (!(bq > 0.f)) return (state ? fmaf(et, ixe, acc) : acc) / den;
+      if (!(bq > 0.f)) return lin_read(bq, (state ? fmaf(et, ixe, acc) : acc) / den);
       const float la = acc == 0.f ? -INFINITY : m + logf(acc);
       const float lb = ixe == 0.f ? -INFINITY : w.mu[task * dp + j] + gt + logf(ixe);
       const float hi = fmaxf(la, lb), lo = fminf(la, lb);
@@ -512,13 +593,13 @@ __global__ void __launch_bounds__(kThreads, 3)
       if (__popc(fm) >= 4) {
         const int j = j0 + half * 32 + lane;
         const bool on = (fm >> lane) & 1u;  // below d
-        const float bq = on ? beta[static_cast<size_t>((h0 + hd) % H) * d + j] : 0.f;
+        const float bq = on ? s_b[j - j0] : 0.f;
         const float *vc = v + r0 * d + (on ? j : 0);
         float m = -INFINITY, acc = 0.f, ixe = 0.f;
         for (int i = 0; i <= t; ++i) m = fmaxf(m, fmaf(bq, __ldg(vc + static_cast<size_t>(i) * d), s_dg[i]));
         for (int i = 0; i <= t; ++i) {
           const float xv = __ldg(vc + static_cast<size_t>(i) * d), y = fmaf(bq, xv, s_dg[i]);
-          const float e = bq > 0.f ? expf(y - m) : expf(s_dg[i]) * xv;
+          const float e = bq > 0.f ? expf(y - m) : expf(s_dg[i]) * lin_value(bq, xv);
           if (!(bq > 0.f) || y != -INFINITY) acc = fmaf(s_sc[i], e, acc);
         }
         if (state && on)
@@ -529,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 3)
       while (fm) {
         const int j = j0 + half * 32 + __ffs(fm) - 1;
         fm &= fm - 1;
-        const float bq = beta[static_cast<size_t>((h0 + hd) % H) * d + j];
+        const float bq = s_b[j - j0];
         float y[2], m = -INFINITY, acc = 0.f, ixe = 0.f;
 #pragma unroll
         for (int k2 = 0; k2 < 2; ++k2) {
@@ -537,7 +618,7 @@ __global__ void __launch_bounds__(kThreads, 3)
           const float xv = i <= t ? __ldg(v + (r0 + i) * d + j) : 0.f;
           y[k2] = i <= t ? fmaf(bq, xv, dg[k2]) : -INFINITY;
           m = fmaxf(m, y[k2]);
-          if (!(bq > 0.f) && i <= t) acc = fmaf(sc[k2] * expf(dg[k2]), xv, acc);
+          if (!(bq > 0.f) && i <= t) acc = fmaf(sc[k2] * expf(dg[k2]), lin_value(bq, xv), acc);
         }
         if (state)
           for (int f = lane; f < M; f += 32) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
@@ -570,7 +651,7 @@ struct GlaPlan {
 GlaPlan gla_plan(long long BH, int T, int m, int d, size_t cap, float *base, GlaWs *w) {
   const int n_ch = (T + kSteps - 1) / kSteps, dp = (d + kCh - 1) / kCh * kCh;
   if (n_ch == 1) return {static_cast<int>(BH < 65535 ? BH : 65535), 1, 0};
-  const size_t per = static_cast<size_t>(m) * dp + m + 2 * dp + 1, head = static_cast<size_t>(m) * dp + m + dp;
+  const size_t per = static_cast<size_t>(m) * dp + m + 2 * dp + 1, head = static_cast<size_t>(m) * dp + m + 2 * dp;
   const size_t room = cap / sizeof(float) / per;
   GlaPlan p;
   if (room >= static_cast<size_t>(n_ch)) {
@@ -596,7 +677,8 @@ GlaPlan gla_plan(long long BH, int T, int m, int d, size_t cap, float *base, Gla
   l.lam = take(n * dp);
   l.mu = take(n * dp);
   l.gl = take(n);
-  l.carry = take(static_cast<size_t>(p.heads) * head);
+  l.eb = take(static_cast<size_t>(p.heads) * dp);
+  l.carry = take(static_cast<size_t>(p.heads) * (head - dp));
   p.floats = o;
   if (w) *w = l;
   return p;
@@ -606,7 +688,9 @@ template <int M>
 cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v, const float *logdecay, const float *beta,
                          float *out, float *logz, int BH, int H, int T, int d, size_t cap, void *ws, cudaStream_t stream) {
   constexpr int kBytes = OutF32<M>::kFloats * 4;
-  cudaError_t e = cudaFuncSetAttribute(gla_out_f32_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
+  const bool lone = T <= kSteps;
+  const auto out_kernel = lone ? gla_out_f32_kernel<M, true> : gla_out_f32_kernel<M, false>;
+  cudaError_t e = cudaFuncSetAttribute(out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBytes);
   if (e != cudaSuccess) return e;
   GlaWs w = {};
   const GlaPlan p = gla_plan(BH, T, M, d, cap, static_cast<float *>(ws), &w);
@@ -615,18 +699,20 @@ cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v, const
   const int vec_o = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   for (int h0 = 0; h0 < BH; h0 += p.heads) {
     const int nh = BH - h0 < p.heads ? BH - h0 : p.heads;
+    if (n_ch > 1) gla_form_f32_kernel<<<dim3(nh, groups), kThreads, 0, stream>>>(v, beta, h0, H, T, d, dp, vec, w);
     for (int c0 = 0; c0 < n_ch; c0 += p.chunks) {
       const int n = n_ch - c0 < p.chunks ? n_ch - c0 : p.chunks;
       if (n_ch > 1) {
         // the sequence's last chunk starts no other: what the scan reads in its slot goes nowhere
         const int own = c0 + n == n_ch ? n - 1 : n;
         if (own > 0)
-          gla_local_f32_kernel<M><<<dim3(own, groups, nh), kThreads, 0, stream>>>(kf, v, logdecay, beta, h0, H, T, d, dp,
-                                                                                  c0, p.chunks, vec, w);
-        gla_scan_f32_kernel<<<dim3((M * dp + M + 255) / 256, nh), 256, 0, stream>>>(beta, h0, H, d, dp, M, c0 == 0 ? 1 : 0,
-                                                                                    n, p.chunks, w);
+          e = launch_kernel(gla_local_f32_kernel<M>, dim3(own, groups, nh), dim3(kThreads), 0, stream, c0 == 0, kf, v,
+                            logdecay, h0, T, d, dp, c0, p.chunks, vec, w);
+        if (e != cudaSuccess) return e;
+        gla_scan_f32_kernel<<<dim3((M * dp + M + 255) / 256, nh), 256, 0, stream>>>(d, dp, M, c0 == 0 ? 1 : 0, n,
+                                                                                    p.chunks, w);
       }
-      gla_out_f32_kernel<M><<<dim3(n, groups, nh), kThreads, kBytes, stream>>>(qf, kf, v, logdecay, beta, out, logz, h0, H,
+      out_kernel<<<dim3(n, groups, nh), kThreads, kBytes, stream>>>(qf, kf, v, logdecay, beta, out, logz, h0, H,
                                                                                T, d, dp, c0, p.chunks, vec, vec_o, w);
     }
   }
