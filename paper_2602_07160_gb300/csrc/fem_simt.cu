@@ -230,10 +230,13 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
 // thread = channel j and key group g (C channels, 128 / C groups): the channel's largest value, then
 // sums at it over the group's keys, the groups combined through shared memory.
 //   L = sum_i P_i,  A_j = sum_i P_i exp(beta_j (v_ij - c_j)),  X_j = sum_i P_i expm1(beta_j (v_ij - c_j))
-// (X of the plain differences at beta = 0), read as above with X = beta W.  What bounds it is latency: one
+// (X of the plain differences at beta = 0), read as above with X = beta W.  An A / L below kSumGuard or not
+// finite (fp32's range could then hide terms that count: the largest value under a tiny weight) is summed
+// again around the largest s_i + beta v_i.  What bounds it is latency: one
 // round of loads, two block reductions and a group's exponentials.  us in a graph, four warps folding key
 // after key / this: B1 H1 T64 d16 12.5 / 4.9, B1 H1 T40 d128 26.9 / 9.4, B4 H8 T47 d64 32.1 / 14.3, B16 H4
 // T30 d128 49.7 / 21.0, B1 H1 T5 d16 3.8 / 3.2.
+constexpr float kSumGuard = 0x1p-84f;
 constexpr int kRowThreads = 128, kRowMaxKeys = 128;
 constexpr size_t kRowSmem = 48 * 1024 - 4096;  // beside the static arrays, without an opt-in
 
@@ -250,7 +253,7 @@ __global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restri
                                                                float *__restrict__ lse, int H, int T, int d, int C,
                                                                int causal) {
   extern __shared__ float simt_smem[];
-  __shared__ float s_p[kRowMaxKeys], s_red[2][4], s_g[3][kRowThreads];
+  __shared__ float s_p[kRowMaxKeys], s_s[kRowMaxKeys], s_red[2][4], s_g[3][kRowThreads];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long row = blockIdx.x, bh = row / T;
   const int t = static_cast<int>(row % T), n = causal ? t + 1 : T, ldk = d + 1;
@@ -285,6 +288,7 @@ __global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restri
   m = fmaxf(fmaxf(s_red[0][0], s_red[0][1]), fmaxf(s_red[0][2], s_red[0][3]));
   float p = tid < n ? expf(s - m) : 0.f;
   s_p[tid] = p;
+  s_s[tid] = s;
 #pragma unroll
   for (int off = 16; off; off >>= 1) p += __shfl_xor_sync(0xffffffffu, p, off);
   if (lane == 0) s_red[1][warp] = p;
@@ -320,8 +324,15 @@ __global__ void __launch_bounds__(kRowThreads) fem_row_kernel(const In *__restri
         A += s_g[1][u * C + jl];
         X += s_g[2][u * C + jl];
       }
-      const float z = X / L;
-      out[row * d + j] = b == 0.f ? c + z : z > -0.5f ? c + log1pf(z) / b : c + logf(A / L) / b;
+      const float z = X / L, r = A / L;
+      float o = b == 0.f ? c + z : z > -0.5f ? c + log1pf(z) / b : c + logf(r) / b;
+      if (b != 0.f && !(z > -0.5f) && !(r >= kSumGuard && r < INFINITY)) {
+        float top = -INFINITY, sum = 0.f;
+        for (int i = 0; i < n; ++i) top = fmaxf(top, fmaf(b, sv[i * d + j], s_s[i]));
+        for (int i = 0; i < n; ++i) sum += expf(fmaf(b, sv[i * d + j], s_s[i]) - top);
+        o = ((top - m) + (logf(sum) - logf(L))) / b;
+      }
+      out[row * d + j] = o;
     }
     if (j0 == 0 && tid == 0 && lse) lse[row] = m + logf(L);
   }

@@ -1,0 +1,37 @@
+"""The fp32 read on the GPU (needs a GB300) where a prior's weights and the tilt leave fp32's
+range on either side: the key with the largest value has a weight that underflows, and the
+keys with weight lie below it by more nats than fp32 holds.
+
+The fp32 read's bound, 1e-4, against the float64 oracle.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_07160_gb300 import build, fem
+from paper_2602_07160_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    build.build()
+    return fem.load()
+
+
+def _check(B, H, T, d, causal):
+    q, k, v, beta = W.make_custom(B, H, T, d, dtype="f32", beta_lo=2.0, beta_hi=1000.0, seed=T + d)
+    q, k = q * 6, k * 6  # scores spread over some hundreds of nats
+    beta[:, 0] = 0.0
+    out, lse = fem.fem_fwd_f32(*(x.cuda() for x in (q, k, v, beta)), causal=causal)
+    fem.check_device_error()
+    ref, ref_lse = oracle.fem_read(q, k, v, beta, causal)
+    assert np.abs(out.cpu().double().numpy() - ref).max() <= 1e-4
+    assert np.abs(lse.cpu().double().numpy() - ref_lse).max() <= 1e-4
+
+
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("T,d", [(3, 1), (33, 16), (64, 20), (128, 40), (70, 64)])
+def test_short_rows(T, d, causal):
+    _check(1, 2, T, d, causal)
