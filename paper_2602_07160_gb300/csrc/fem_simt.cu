@@ -22,13 +22,17 @@
 //   o = c + log1p(beta W / L) / beta   when beta W / L > -1/2 (no cancellation),
 //   o = c + log(A / L) / beta          otherwise,
 //   o = c + W / L                      at beta = 0 (the prior mean),
-// which is (1/beta) log sum_i p_t(i) exp(beta v_ij) (Sec. 2.3).
+// which is (1/beta) log sum_i p_t(i) exp(beta v_ij) (Sec. 2.3).  An A / L below kSumGuard or not finite
+// (fp32's range could then hide terms that count: the largest value under a tiny weight) is summed again
+// around the largest s_i + beta v_i.
 #include "fem_common.cuh"
 #include "fem_launch.h"
 
 namespace fem {
 
 constexpr int kSimtMaxPerLane = 8;  // d <= 256
+
+constexpr float kSumGuard = 0x1p-84f;
 
 // rows up to which a row gets a block of its own (its keys split over the warps)
 constexpr long long kSimtSplitRows = 2048;
@@ -46,6 +50,46 @@ __device__ __forceinline__ float expm1_over_beta(float b, float x) {
 
 __device__ __forceinline__ float ld_in(const float *p) { return *p; }
 __device__ __forceinline__ float ld_in(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+
+// The warp's row again for the channel slots of `redo` (a mask per lane): the keys in turn, first for the
+// largest s_i + beta v_i, then for the sum around it.
+template <typename In, int PER>
+__device__ __noinline__ void simt_exact(const In *qr, const In *kb, const In *vb, const float *beta, int n, int d,
+                                        float m, float L, unsigned redo, float *orow) {
+  const int lane = threadIdx.x & 31;
+  const float inv_sqrt_d = rsqrtf(static_cast<float>(d));
+  float top[PER], sum[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    top[u] = -INFINITY;
+    sum[u] = 0.f;
+  }
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i = 0; i < n; ++i) {
+      const In *kr = kb + static_cast<long long>(i) * d, *vr = vb + static_cast<long long>(i) * d;
+      float s = 0.f;
+      for (int j = lane; j < d; j += 32) s = fmaf(ld_in(qr + j), ld_in(kr + j), s);
+#pragma unroll
+      for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      s *= inv_sqrt_d;
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        if (!((redo >> u) & 1u)) continue;
+        const int j = lane + 32 * u;
+        const float y = fmaf(beta[j], ld_in(vr + j), s);
+        if (pass == 0)
+          top[u] = fmaxf(top[u], y);
+        else
+          sum[u] += expf(y - top[u]);
+      }
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int j = lane + 32 * u;
+    if ((redo >> u) & 1u) orow[j] = ((top[u] - m) + (logf(sum[u]) - logf(L))) / beta[j];
+  }
+}
 
 // PER: channel slots per lane, d <= 32 PER (the unrolled per-slot code costs
 // issue slots even where a slot is empty).  SPLIT (few rows): one row per
@@ -208,6 +252,7 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
   }
   if (!valid) return;
 
+  unsigned redo = 0;
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int j = lane + 32 * u;
@@ -217,11 +262,14 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
     if (b == 0.f) {
       o = c[u] + W[u] / L;
     } else {
-      const float z = b * W[u] / L;
-      o = z > -0.5f ? c[u] + log1pf(z) / b : c[u] + logf(A[u] / L) / b;
+      const float z = b * W[u] / L, r = A[u] / L;
+      o = z > -0.5f ? c[u] + log1pf(z) / b : c[u] + logf(r) / b;
+      if (!(z > -0.5f) && !(r >= kSumGuard && r < INFINITY)) redo |= 1u << u;
     }
-    out[row * d + j] = o;
+    if (!((redo >> u) & 1u)) out[row * d + j] = o;
   }
+  if (__any_sync(0xffffffffu, redo != 0u))
+    simt_exact<In, PER>(q + row * d, kb, vb, beta + static_cast<size_t>(h) * d, n, d, m, L, redo, out + row * d);
   if (lse && lane == 0) lse[row] = m + logf(L);
 }
 
@@ -230,13 +278,11 @@ __global__ void __launch_bounds__(128) fem_simt_kernel(const In *__restrict__ q,
 // thread = channel j and key group g (C channels, 128 / C groups): the channel's largest value, then
 // sums at it over the group's keys, the groups combined through shared memory.
 //   L = sum_i P_i,  A_j = sum_i P_i exp(beta_j (v_ij - c_j)),  X_j = sum_i P_i expm1(beta_j (v_ij - c_j))
-// (X of the plain differences at beta = 0), read as above with X = beta W.  An A / L below kSumGuard or not
-// finite (fp32's range could then hide terms that count: the largest value under a tiny weight) is summed
-// again around the largest s_i + beta v_i.  What bounds it is latency: one
+// (X of the plain differences at beta = 0), read as above with X = beta W, a rejected A / L summed again
+// likewise.  What bounds it is latency: one
 // round of loads, two block reductions and a group's exponentials.  us in a graph, four warps folding key
 // after key / this: B1 H1 T64 d16 12.5 / 4.9, B1 H1 T40 d128 26.9 / 9.4, B4 H8 T47 d64 32.1 / 14.3, B16 H4
 // T30 d128 49.7 / 21.0, B1 H1 T5 d16 3.8 / 3.2.
-constexpr float kSumGuard = 0x1p-84f;
 constexpr int kRowThreads = 128, kRowMaxKeys = 128;
 constexpr size_t kRowSmem = 48 * 1024 - 4096;  // beside the static arrays, without an opt-in
 

@@ -35,3 +35,9 @@ def _check(B, H, T, d, causal):
 @pytest.mark.parametrize("T,d", [(3, 1), (33, 16), (64, 20), (128, 40), (70, 64)])
 def test_short_rows(T, d, causal):
     _check(1, 2, T, d, causal)
+
+
+@pytest.mark.parametrize("B,H,T,d", [(1, 2, 33, 200), (3, 1, 128, 129), (1, 1, 130, 256), (80, 1, 28, 33), (300, 1, 9, 100)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_rows_by_warps(B, H, T, d, causal):
+    _check(B, H, T, d, causal)
