@@ -461,6 +461,7 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
     }
   }
   // ---- the entries to evaluate again, one at a time by the whole warp
+  __syncwarp();  // their first values, stored by their own threads, come before lane 0's
 #pragma unroll 1
   for (int c = 0; c < NC; ++c) {
     unsigned mine = 0u;
