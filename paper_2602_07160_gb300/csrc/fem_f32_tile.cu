@@ -317,13 +317,16 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
         }
       }
     }
+    float m0[4];  // the row's shift, 0 while no score of the row is above -inf (its weights are then 0)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) m0[r] = m[r] == -INFINITY ? 0.f : m[r];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       float p[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const float x = (r & 1) ? s[r >> 1][c].y : s[r >> 1][c].x;
-        const float tm = x - m[r];
+        const float tm = x - m0[r];
         p[r] = tm < -60.f ? expf(tm + 40.f * kLn2) : expf(tm) * kWeightScale;
         l[r] += p[r];
       }

@@ -41,3 +41,19 @@ def test_short_rows(T, d, causal):
 @pytest.mark.parametrize("causal", [True, False])
 def test_rows_by_warps(B, H, T, d, causal):
     _check(B, H, T, d, causal)
+
+
+@pytest.mark.parametrize("T,first,last,causal", [(192, 64, 128, False), (200, 0, 64, False), (300, 70, 300, True), (60, 10, 30, True)])
+def test_keys_with_a_score_of_minus_infinity(T, first, last, causal):
+    """Keys masked by a score of -inf, whole tiles of them among those: no weight, for the read and
+    for its log-normaliser (in the oracle their scores are some -1e5)."""
+    q, k, v, beta = W.make_custom(1, 1, T, 16, dtype="f32", seed=T)
+    q = q.abs() + 0.1
+    far = k.clone()
+    far[:, :, first:last] = -1e5
+    k[:, :, first:last] = -float("inf")
+    out, lse = fem.fem_fwd_f32(*(x.cuda() for x in (q, k, v, beta)), causal=causal)
+    fem.check_device_error()
+    ref, ref_lse = oracle.fem_read(q, far, v, beta, causal)
+    assert np.abs(out.cpu().double().numpy() - ref).max() <= 1e-4
+    assert np.abs(lse.cpu().double().numpy() - ref_lse).max() <= 1e-4
