@@ -24,8 +24,9 @@
 // reach 2^52 (with the row maximum's lag), bank entries 2^52, their sums 2^119 at 2^15 keys, and
 // what the range can drop from a sum (2^-126 of either's largest) stays below 2^-24 of an A / L of
 // kTileGuard.  An entry whose A / L is not finite or lies below that (peaked priors, wide spans,
-// infinities among the values of keys the row does not see) is evaluated again key by key, from the
-// keys the row sees alone.  Every product and sum is fp32, as in fem_simt.cu.
+// infinities among the values of keys the row does not see) is summed again around its own largest
+// s_i + beta v_i, the key tiles once more (sweep_again); one of a linear channel, which only values
+// that are not finite can reject, key by key.  Every product and sum is fp32, as in fem_simt.cu.
 //
 // Layout: two groups of 256 threads take the key tiles in turn, each with its own K, bank and P
 // tiles in shared memory and its own accumulators (the heaviest block's chain is half as long, and
@@ -35,6 +36,8 @@
 // 31 %: a warp waits out every dependent pair).  K and Q lie transposed ([channel][row]); P's
 // 16-byte chunks are swizzled by key so its transposed stores spread over the banks.  Up to 64
 // channels the next tile's K and V rows are loaded into registers ahead of the contractions.
+#include <type_traits>
+
 #include "fem_common.cuh"
 #include "fem_f32.cuh"
 #include "fem_launch.h"
@@ -57,9 +60,11 @@ struct TileLay {
   static constexpr int kGroupFloats = DP * kTLd + kTK * kEl + kTK * kTR;
   static constexpr int kPar = DP * kTLd + kGroups * kGroupFloats;  // per channel: beta, 1/beta, c, linear
   static constexpr int kRed = kPar + 4 * DP;                 // the groups' m and L for the merge
-  static constexpr int kFloats = kRed + kGroups * kTR * 2;
+  static constexpr int kAny = kRed + kGroups * kTR * 2;      // per thread of a group: entries to sum again
+  static constexpr int kFloats = kAny + kGT;
   static constexpr int kBytes = kFloats * 4;
   static_assert(kBytes <= 227 * 1024, "shared memory");
+  static_assert(2 * kTR * DP <= kGroupFloats, "a group's state of the second sweep fits its tiles");
   static_assert(4 * (kGroups * kGT / (DP / 4)) * DP <= kGroups * kGroupFloats, "statistics' partials fit the tiles");
 };
 
@@ -103,6 +108,174 @@ __device__ __noinline__ float read_exact(const In *qr, const In *kb, const In *v
   if (b == 0.f) return c + W / L;
   const float z = b * W / L;
   return z > -0.5f ? c + log1pf(z) / b : ((top - m) + (logf(A) - logf(L))) / b;
+}
+
+// The block's key tiles once more for the rejected entries of shifted channels (Lay::kAny: bit 4 c + r of a
+// thread's word is row 4 ty + r, channel chan(c)): scores as before, then in warps that have any the largest
+// s_i + beta v_i of the tile and the sum around the running one.  What bounds it is the issue of the tile's
+// (row, key, channel) terms and their exponentials.  Entry by entry, scores and all, a warp spent some 40 us on each at
+// T2048 d64 and peaked priors reject most of them: B1 H4 T2048 d64 causal, scores of deviation 16, beta 10 to
+// 100 73.5 ms (the warp-per-row form 2.5, with -inf for many); now 0.53 ms.
+template <typename In, int DP>
+__device__ __noinline__ void sweep_again(float *smem, const In *kb, const In *vb, float *ob, int T, int d, int t0,
+                                         int n_keys, int causal) {
+  using Lay = TileLay<DP>;
+  constexpr int NC = DP / 16, kEl = Lay::kEl, CQ = DP / 4;
+  const int tid = threadIdx.x, g = tid / kGT, gt = tid % kGT, ty = gt >> 4, tx = gt & 15;
+  float *sQ = smem, *sK = smem + DP * kTLd + g * Lay::kGroupFloats, *sV = sK + DP * kTLd, *sS = sV + kTK * kEl;
+  const float *pB = smem + Lay::kPar, *sRed = smem + Lay::kRed;
+  const unsigned mask = reinterpret_cast<const unsigned *>(smem + Lay::kAny)[gt];
+  const bool any = __any_sync(0xffffffffu, mask != 0u);
+  const bool vec = (d & 3) == 0;
+  const float scale = kLog2e * rsqrtf(static_cast<float>(d));
+  auto chan = [&](int c) { return NC == 2 ? tx * 2 + c : (c >> 2) * 64 + tx * 4 + (c & 3); };
+  float b[NC];
+  float2 top[2][NC], A[2][NC];  // rows 2 u, 2 u + 1 of the thread's four; exponents in units of ln 2
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    b[c] = pB[chan(c)] * kLog2e;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      top[u][c] = make_float2(-INFINITY, -INFINITY);
+      A[u][c] = make_float2(0.f, 0.f);
+    }
+  }
+  const int n_kt = (n_keys + kTK - 1) / kTK;
+  for (int kt = g; kt < n_kt; kt += kGroups) {
+    const int k0 = kt * kTK, nk = min(kTK, n_keys - k0);
+    bar_sync(1 + g, kGT);  // the previous tile is consumed
+#pragma unroll 4
+    for (int e = gt; e < kTK * CQ; e += kGT) {
+      const int r = e % kTK, j = (e / kTK) * 4;
+      const float4 k4 = r < nk ? ld_row4(kb + static_cast<size_t>(k0 + r) * d, j, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      sK[j * kTLd + r] = k4.x;
+      sK[(j + 1) * kTLd + r] = k4.y;
+      sK[(j + 2) * kTLd + r] = k4.z;
+      sK[(j + 3) * kTLd + r] = k4.w;
+      const int rv = e / CQ, jv = (e % CQ) * 4;
+      *reinterpret_cast<float4 *>(sV + rv * kEl + jv) =
+          rv < nk ? ld_row4(vb + static_cast<size_t>(k0 + rv) * d, jv, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    bar_sync(1 + g, kGT);
+    float2 s[2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) s[i][c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int e = 0; e < DP; ++e) {
+      const float4 a = ld4(sQ + e * kTLd + ty * 4), k4 = ld4(sK + e * kTLd + tx * 4);
+      const float2 ar[2] = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
+      const float kr[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) s[i][c] = __ffma2_rn(ar[i], make_float2(kr[c], kr[c]), s[i][c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float x[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int lim = causal ? min(nk, t0 + ty * 4 + r + 1 - k0) : nk;
+        x[r] = ((r & 1) ? s[r >> 1][c].y : s[r >> 1][c].x) * scale;
+        if (tx * 4 + c >= lim) x[r] = -INFINITY;
+      }
+      *reinterpret_cast<float4 *>(sS + (tx * 4 + c) * kTR + ((ty ^ tx) << 2)) = make_float4(x[0], x[1], x[2], x[3]);
+    }
+    bar_sync(1 + g, kGT);
+    if (!any) continue;
+    float2 was[2][NC];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) was[i][c] = top[i][c];
+    // s_i + beta v_i of key i; masked: -inf whatever the value, which may not be finite
+    auto terms = [&](int i, float2 (&y)[2][NC], bool masked) {
+      const float4 a = ld4(sS + i * kTR + ((ty ^ (i >> 2)) << 2));
+      const float2 sr[2] = {make_float2(a.x, a.y), make_float2(a.z, a.w)};
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const float v = sV[i * kEl + chan(c)];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          y[u][c] = __ffma2_rn(make_float2(b[c], b[c]), make_float2(v, v), sr[u]);
+          if (masked) {
+            if (sr[u].x == -INFINITY) y[u][c].x = -INFINITY;
+            if (sr[u].y == -INFINITY) y[u][c].y = -INFINITY;
+          }
+        }
+      }
+    };
+    auto sweep = [&](auto ragged) {
+      constexpr bool kMasked = decltype(ragged)::value;
+#pragma unroll 2
+      for (int i = 0; i < nk; ++i) {
+        float2 y[2][NC];
+        terms(i, y, kMasked);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int c = 0; c < NC; ++c)
+            top[u][c] = make_float2(fmaxf(top[u][c].x, y[u][c].x), fmaxf(top[u][c].y, y[u][c].y));
+      }
+      float2 neg[2][NC];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const float2 t = top[u][c], w = was[u][c];
+          A[u][c] = make_float2(t.x > w.x ? A[u][c].x * ex2_approx(w.x - t.x) : A[u][c].x,
+                                t.y > w.y ? A[u][c].y * ex2_approx(w.y - t.y) : A[u][c].y);
+          // no finite term yet: every exponential below is that of -inf
+          neg[u][c] = make_float2(t.x == -INFINITY ? 0.f : -t.x, t.y == -INFINITY ? 0.f : -t.y);
+        }
+#pragma unroll 2
+      for (int i = 0; i < nk; ++i) {
+        float2 y[2][NC];
+        terms(i, y, kMasked);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            const float2 x = __fadd2_rn(y[u][c], neg[u][c]);
+            A[u][c] = __fadd2_rn(A[u][c], make_float2(ex2_approx(x.x), ex2_approx(x.y)));
+          }
+      }
+    };
+    if (causal && k0 + kTK > t0 + 1)
+      sweep(std::true_type());
+    else
+      sweep(std::false_type());
+  }
+  // the groups' states merged by the first
+  bar_sync(1 + g, kGT);
+  float *st = smem + DP * kTLd + Lay::kGroupFloats;  // the second group's tiles: [64][DP] top, then A
+  auto of_row = [](const float2 (&x)[2][NC], int r, int c) { return (r & 1) ? x[r >> 1][c].y : x[r >> 1][c].x; };
+  if (g > 0 && any) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        st[(ty * 4 + r) * DP + chan(c)] = of_row(top, r, c);
+        st[(kTR + ty * 4 + r) * DP + chan(c)] = of_row(A, r, c);
+      }
+  }
+  __syncthreads();
+  if (g > 0 || !mask) return;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int row = ty * 4 + r;
+    const float m = sRed[row * 2], ll = logf(sRed[row * 2 + 1]);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (!((mask >> (4 * c + r)) & 1u)) continue;
+      const float t1 = of_row(top, r, c), t2 = st[row * DP + chan(c)], tn = fmaxf(t1, t2);
+      const float sum = (t1 == -INFINITY ? 0.f : of_row(A, r, c) * ex2_approx(t1 - tn)) +
+                        (t2 == -INFINITY ? 0.f : st[(kTR + row) * DP + chan(c)] * ex2_approx(t2 - tn));
+      ob[static_cast<size_t>(t0 + row) * d + chan(c)] = (fmaf(tn, kLn2, -m) + (logf(sum) - ll)) / pB[chan(c)];
+    }
+  }
 }
 
 template <typename In, int DP>
@@ -387,104 +560,121 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
     }
   }
   __syncthreads();
-  if (g > 0) return;
-  for (int og = 1; og < kGroups; ++og) {
-    const float *st = tile_smem + DP * kTLd + og * Lay::kGroupFloats;
+  unsigned again = 0;  // entries of shifted channels to sum again: bit 4 c + r
+  if (g == 0) {
+    for (int og = 1; og < kGroups; ++og) {
+      const float *st = tile_smem + DP * kTLd + og * Lay::kGroupFloats;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float m2 = sRed[(og * kTR + ty * 4 + r) * 2], l2 = sRed[(og * kTR + ty * 4 + r) * 2 + 1];
-      const float mn = fmaxf(m[r], m2);
-      const float a1 = m[r] == -INFINITY ? 0.f : expf(m[r] - mn), a2 = m2 == -INFINITY ? 0.f : expf(m2 - mn);
-      l[r] = l[r] * a1 + l2 * a2;
+      for (int r = 0; r < 4; ++r) {
+        const float m2 = sRed[(og * kTR + ty * 4 + r) * 2], l2 = sRed[(og * kTR + ty * 4 + r) * 2 + 1];
+        const float mn = fmaxf(m[r], m2);
+        const float a1 = m[r] == -INFINITY ? 0.f : expf(m[r] - mn), a2 = m2 == -INFINITY ? 0.f : expf(m2 - mn);
+        l[r] = l[r] * a1 + l2 * a2;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        float &a = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
-        a = a * a1 + st[(ty * 4 + r) * DP + chan(c)] * a2;
-      }
-      m[r] = mn;
-    }
-  }
-  // ---- the read
-  unsigned redo[NC];  // per channel: the rows to evaluate again
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    redo[c] = 0u;
-    const int j = chan(c);
-    const float b = pB[j], ib = pI[j], cc = pC[j];
-    const bool lin = pL[j] != 0.f;
-    const float ib_lo = b > 0.f ? fmaf(-b, ib, 1.f) * ib : 0.f;  // 1 / b is ib + ib_lo
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      float &a = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
-      const float x = a / l[r];
-      const bool bad = lin ? !(b * x > -0.9f && fabsf(x) < INFINITY) : !(x > kTileGuard && x < INFINITY);
-      if (bad && j < d && t0 + ty * 4 + r < T) redo[c] |= 1u << r;
-      if (b > 0.f) {
-        // log1p(b x) or log(x), the latter as n ln 2 + log(mantissa) in two parts, over b and onto c
-        // with the rounding errors of both steps carried: |c - o| may be several times |o|
-        float hi, lo = 0.f;
-        if (lin) {
-          hi = log1pf(b * x);
-        } else {
-          const int n = ((__float_as_int(x) - 0x3f400000) >> 23);  // the mantissa in [3/4, 3/2)
-          const float f = static_cast<float>(n), lm = logf(__int_as_float(__float_as_int(x) - (n << 23)));
-          hi = f * 0x1.62e4p-1f;  // ln 2 to 16 bits: exact
-          lo = fmaf(f, 0x1.7f7d1cp-20f, lm);
+        for (int c = 0; c < NC; ++c) {
+          float &a = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
+          a = a * a1 + st[(ty * 4 + r) * DP + chan(c)] * a2;
         }
-        const float t = hi + lo, tlo = lo - (t - hi), qv = t * ib, qlo = fmaf(t, ib, -qv) + fmaf(tlo, ib, t * ib_lo);
-        const float o = cc + qv, z = o - cc;
-        a = o + (((cc - (o - z)) + (qv - z)) + qlo);
+        m[r] = mn;
+      }
+    }
+    // ---- the read
+    unsigned redo[NC];  // per channel: the rows to evaluate again
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      redo[c] = 0u;
+      const int j = chan(c);
+      const float b = pB[j], ib = pI[j], cc = pC[j];
+      const bool lin = pL[j] != 0.f;
+      const float ib_lo = b > 0.f ? fmaf(-b, ib, 1.f) * ib : 0.f;  // 1 / b is ib + ib_lo
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float &a = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
+        const float x = a / l[r];
+        const bool bad = lin ? !(b * x > -0.9f && fabsf(x) < INFINITY) : !(x > kTileGuard && x < INFINITY);
+        if (bad && j < d && t0 + ty * 4 + r < T) {
+          if (lin)
+            redo[c] |= 1u << r;
+          else
+            again |= 1u << (4 * c + r);
+        }
+        if (b > 0.f) {
+          // log1p(b x) or log(x), the latter as n ln 2 + log(mantissa) in two parts, over b and onto c
+          // with the rounding errors of both steps carried: |c - o| may be several times |o|
+          float hi, lo = 0.f;
+          if (lin) {
+            hi = log1pf(b * x);
+          } else {
+            const int n = ((__float_as_int(x) - 0x3f400000) >> 23);  // the mantissa in [3/4, 3/2)
+            const float f = static_cast<float>(n), lm = logf(__int_as_float(__float_as_int(x) - (n << 23)));
+            hi = f * 0x1.62e4p-1f;  // ln 2 to 16 bits: exact
+            lo = fmaf(f, 0x1.7f7d1cp-20f, lm);
+          }
+          const float t = hi + lo, tlo = lo - (t - hi), qv = t * ib, qlo = fmaf(t, ib, -qv) + fmaf(tlo, ib, t * ib_lo);
+          const float o = cc + qv, z = o - cc;
+          a = o + (((cc - (o - z)) + (qv - z)) + qlo);
+        } else {
+          a = cc + x;
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int t = t0 + ty * 4 + r;
+      if (t >= T) continue;
+      float *o = out + (bh * T + t) * d;
+      if (lse && tx == 0) lse[bh * T + t] = m[r] + logf(l[r] * (1.f / kWeightScale));
+      if constexpr (NC == 2) {
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          if (chan(c) < d) o[chan(c)] = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
       } else {
-        a = cc + x;
+#pragma unroll
+        for (int c = 0; c < NC; c += 4) {
+          float x[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[u] = (r & 1) ? acc[r >> 1][c + u].y : acc[r >> 1][c + u].x;
+          if (vec && chan(c) < d) *reinterpret_cast<float4 *>(o + chan(c)) = make_float4(x[0], x[1], x[2], x[3]);
+          if (!vec)
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (chan(c + u) < d) o[chan(c + u)] = x[u];
+        }
       }
     }
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int t = t0 + ty * 4 + r;
-    if (t >= T) continue;
-    float *o = out + (bh * T + t) * d;
-    if (lse && tx == 0) lse[bh * T + t] = m[r] + logf(l[r] * (1.f / kWeightScale));
-    if constexpr (NC == 2) {
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-        if (chan(c) < d) o[chan(c)] = (r & 1) ? acc[r >> 1][c].y : acc[r >> 1][c].x;
-    } else {
-#pragma unroll
-      for (int c = 0; c < NC; c += 4) {
-        float x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = (r & 1) ? acc[r >> 1][c + u].y : acc[r >> 1][c + u].x;
-        if (vec && chan(c) < d) *reinterpret_cast<float4 *>(o + chan(c)) = make_float4(x[0], x[1], x[2], x[3]);
-        if (!vec)
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (chan(c + u) < d) o[chan(c + u)] = x[u];
-      }
-    }
-  }
-  // ---- the entries to evaluate again, one at a time by the whole warp
-  __syncwarp();  // their first values, stored by their own threads, come before lane 0's
+    // ---- the linear channels' entries to evaluate again, one at a time by the whole warp
+    __syncwarp();  // their first values, stored by their own threads, come before lane 0's
 #pragma unroll 1
-  for (int c = 0; c < NC; ++c) {
-    unsigned mine = 0u;
+    for (int c = 0; c < NC; ++c) {
+      unsigned mine = 0u;
 #pragma unroll
-    for (int u = 0; u < NC; ++u) mine = u == c ? redo[u] : mine;
-    unsigned who = __ballot_sync(0xffffffffu, mine != 0u);
-    while (who) {
-      const int src = __ffs(who) - 1;
-      who &= who - 1;
-      unsigned rows = __shfl_sync(0xffffffffu, mine, src);
-      const int j = __shfl_sync(0xffffffffu, chan(c), src), ry = __shfl_sync(0xffffffffu, ty, src);
-      while (rows) {
-        const int t = t0 + ry * 4 + __ffs(rows) - 1;
-        rows &= rows - 1;
-        const float o = read_exact(qb + static_cast<size_t>(t) * d, kb, vb, causal ? t + 1 : T, d, j, pB[j], inv_sqrt_d,
-                                   lane);
-        if (lane == 0) out[(bh * T + t) * d + j] = o;
+      for (int u = 0; u < NC; ++u) mine = u == c ? redo[u] : mine;
+      unsigned who = __ballot_sync(0xffffffffu, mine != 0u);
+      while (who) {
+        const int src = __ffs(who) - 1;
+        who &= who - 1;
+        unsigned rows = __shfl_sync(0xffffffffu, mine, src);
+        const int j = __shfl_sync(0xffffffffu, chan(c), src), ry = __shfl_sync(0xffffffffu, ty, src);
+        while (rows) {
+          const int t = t0 + ry * 4 + __ffs(rows) - 1;
+          rows &= rows - 1;
+          const float o = read_exact(qb + static_cast<size_t>(t) * d, kb, vb, causal ? t + 1 : T, d, j, pB[j], inv_sqrt_d,
+                                     lane);
+          if (lane == 0) out[(bh * T + t) * d + j] = o;
+        }
       }
     }
+    if (tx == 0) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        sRed[(ty * 4 + r) * 2] = m[r];
+        sRed[(ty * 4 + r) * 2 + 1] = l[r] * (1.f / kWeightScale);
+      }
+    }
+    reinterpret_cast<unsigned *>(tile_smem + Lay::kAny)[gt] = again;
   }
+  if (__syncthreads_or(again != 0u))
+    sweep_again<In, DP>(tile_smem, kb, vb, out + bh * T * d, T, d, t0, n_keys, causal);
 }
 
 template <typename In, int DP>

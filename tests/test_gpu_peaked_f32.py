@@ -57,3 +57,17 @@ def test_keys_with_a_score_of_minus_infinity(T, first, last, causal):
     ref, ref_lse = oracle.fem_read(q, far, v, beta, causal)
     assert np.abs(out.cpu().double().numpy() - ref).max() <= 1e-4
     assert np.abs(lse.cpu().double().numpy() - ref_lse).max() <= 1e-4
+
+
+@pytest.mark.parametrize("B,H,T,d", [(1, 2, 129, 16), (1, 1, 200, 128), (2, 1, 90, 64), (1, 1, 333, 33), (1, 1, 700, 60)])
+@pytest.mark.parametrize("causal", [True, False])
+def test_tiles(B, H, T, d, causal):
+    _check(B, H, T, d, causal)
+
+
+def test_tiles_of_bf16_narrow_heads():
+    q, k, v, beta = W.make_custom(1, 2, 300, 32, beta_lo=2.0, beta_hi=1000.0, seed=4)
+    q, k = q * 6, k * 6
+    out, _ = fem.fem_fwd(*(x.cuda() for x in (q, k, v, beta)), causal=True)
+    ref, _ = oracle.fem_read(q, k, v, beta, True)
+    assert np.abs(out.cpu().double().numpy() - ref).max() <= 1e-4
