@@ -56,7 +56,7 @@ __device__ __forceinline__ void bwd_terms(float b, float inv_b, float inv_b2, fl
 // MODE 1: a warp per R consecutive key rows i  -> dk_i and dv_i.
 // Lane l holds channels l + 32 u (u < PER); the R rows share every load of
 // the other side's row and their butterfly sums interleave.
-template <int MODE, int R, int PER>
+template <int MODE, int R, int PER, bool MARKED>
 __global__ void __launch_bounds__(128) fem_bwd_kernel(const float *__restrict__ q, const float *__restrict__ k,
                                                        const float *__restrict__ v, const float *__restrict__ beta,
                                                        const float *__restrict__ out, const float *__restrict__ lse,
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(128) fem_bwd_kernel(const float *__restrict__ 
   if (grp >= n_groups) return;
   const int gpb = (T + R - 1) / R;  // row groups per (b, h)
   const long long bh = grp / gpb;
-  if (peaked && !peaked[bh]) return;  // the head is done (fem_bwd_tile.cu)
+  if (MARKED && !peaked[bh]) return;  // the head is done (fem_bwd_tile.cu)
   const int r0 = static_cast<int>(grp % gpb) * R;
   const int nr = min(R, T - r0);  // rows of this group
   const int h = static_cast<int>(bh % H);
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(128) fem_bwd_kernel(const float *__restrict__ 
       const int j = lane + 32 * u;
       if (j >= d) continue;
       da[base + static_cast<size_t>(r) * d + j] = acc1[w][u] * inv_sqrt_d;
-      if (MODE == 0) atomicAdd(&dbeta[(peaked ? bh : h) * d + j], acc2[w][u]);
+      if (MODE == 0) atomicAdd(&dbeta[(MARKED ? bh : h) * d + j], acc2[w][u]);
       else db[base + static_cast<size_t>(r) * d + j] = acc2[w][u];
     }
   }
@@ -176,10 +176,10 @@ static cudaError_t launch_bwd_rp(const float *q, const float *k, const float *v,
                                  int B, int H, int T, int d, int causal, const int *peaked, cudaStream_t stream) {
   const long long n_groups = static_cast<long long>(B) * H * ((T + R - 1) / R);
   const unsigned blocks = static_cast<unsigned>((n_groups + 3) / 4);
-  fem_bwd_kernel<0, R, PER><<<blocks, 128, 0, stream>>>(q, k, v, beta, out, lse, dout, dq, nullptr, dbeta, H, T, d,
-                                                        causal, n_groups, peaked);
-  fem_bwd_kernel<1, R, PER><<<blocks, 128, 0, stream>>>(q, k, v, beta, out, lse, dout, dk, dv, nullptr, H, T, d,
-                                                        causal, n_groups, peaked);
+  const auto rows = peaked ? fem_bwd_kernel<0, R, PER, true> : fem_bwd_kernel<0, R, PER, false>;
+  const auto keys = peaked ? fem_bwd_kernel<1, R, PER, true> : fem_bwd_kernel<1, R, PER, false>;
+  rows<<<blocks, 128, 0, stream>>>(q, k, v, beta, out, lse, dout, dq, nullptr, dbeta, H, T, d, causal, n_groups, peaked);
+  keys<<<blocks, 128, 0, stream>>>(q, k, v, beta, out, lse, dout, dk, dv, nullptr, H, T, d, causal, n_groups, peaked);
   return cudaGetLastError();
 }
 
@@ -187,9 +187,18 @@ cudaError_t launch_bwd_pairs(const float *q, const float *k, const float *v, con
                              const float *lse, const float *dout, float *dq, float *dk, float *dv, float *dbeta, int B,
                              int H, int T, int d, int causal, const int *peaked,
                              cudaStream_t stream) {
-  // rows per warp: four while a lane holds at most two channels, fewer beyond
 #define FEM_BWD(R, PER) \
   launch_bwd_rp<R, PER>(q, k, v, beta, out, lse, dout, dq, dk, dv, dbeta, B, H, T, d, causal, peaked, stream)
+  // Rows per warp: four while a lane holds at most two channels, fewer beyond, so that a key's row is loaded
+  // for several; one while the rows don't fill the chip, where the warps in flight count (twice as many rows at
+  // 33 to 64 channels).  us, four (two at d 128) / one: B1 H4 T64 d64 102 / 62, B8 H8 T40 d64 72 / 43, B8 H8
+  // T128 d64 259 / 198, B1 H4 T2048 d64 3270 / 2440, B1 H4 T300 d128 387 / 347, B8 H8 T40 d16 49 / 43; beyond
+  // the lines, B16 H4 T300 d64 861 / 885, B4 H4 T300 d128 519 / 583, B16 H4 T1024 d32 4200 / 5260.
+  if (static_cast<long long>(B) * H * T * (d > 32 && d <= 64 ? 1 : 2) <= kBwdFewRows) {
+    if (d <= 32) return FEM_BWD(1, 1);
+    if (d <= 64) return FEM_BWD(1, 2);
+    if (d <= 128) return FEM_BWD(1, 4);
+  }
   if (d <= 32) return FEM_BWD(4, 1);
   if (d <= 64) return FEM_BWD(4, 2);
   if (d <= 128) return FEM_BWD(2, 4);

@@ -24,9 +24,11 @@
 // All exponents carry their rounding errors (exp_tilt), which keeps the gradients'
 // error at that of exp(x) taken directly.  Channels whose spread exceeds that (or is
 // not finite) take no part in the contractions; their terms are formed pair by pair
-// beside them (WideChannels).  Heads where some visible pair's weight falls below
-// e^-60 (its e^x could leave fp32's range) are marked and taken by the kernels of
-// fem_bwd.cu, which form every term from its own exponent.
+// beside them (wide_terms).  A visible pair whose weight falls below e^-60 marks its
+// head (its e^x could leave fp32's range; and where the prior is that peaked, posterior
+// and prior differ so little that the factors' differences lose digits: dbeta 4e-4 off
+// at scores of deviation 64), as does a head with most channels wide; the kernels of
+// fem_bwd.cu, which form every term from its own exponent, take those.
 //
 // What bounds it: issue around the FMA pipe (3 d multiply-adds per pair in the row
 // pass, 5 d in the key pass); fem_bwd.cu's form spends some 50 issue slots a pair and
@@ -49,12 +51,50 @@ constexpr int kBLd = 68;          // leading dimension of a transposed 64-row ti
 constexpr float kWideExp = 72.f;  // largest |a|, |b| of a factored channel: 2^+-104
 constexpr float kPeakLog = -60.f;
 
+// A head's sample of pairs for the mark of peaked priors: warp w takes row T - 1 - w T / 32 and 16 of its keys,
+// lanes over channels.  Without it a marked head pays the row pass's first tiles before its own kernels; what
+// the sample misses is still found there.  us, plain / peaked heads, without and with: B8 H8 T128 d64 100 / 242,
+// 106 / 223, B64 H6 T192 d128 1188 / 2922, 1212 / 2660 (pair by pair alone 2540); below kSampleT it costs the
+// plain ones up to 11 % (B64 H6 T64 d16 94, 105).
+constexpr int kSampleT = 96, kSampleKeys = 16;
+__device__ __forceinline__ bool sample_peaked(const float *q, const float *k, const float *lse, int T, int d, int causal) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = T - 1 - static_cast<int>(static_cast<long long>(warp) * T / 32), n = causal ? t + 1 : T;
+  float s[kSampleKeys];
+#pragma unroll
+  for (int u = 0; u < kSampleKeys; ++u) s[u] = 0.f;
+  for (int j = lane; j < d; j += 32) {
+    const float a = q[static_cast<size_t>(t) * d + j];
+#pragma unroll
+    for (int u = 0; u < kSampleKeys; ++u)
+      s[u] = fmaf(a, k[static_cast<size_t>(static_cast<long long>(u) * n / kSampleKeys) * d + j], s[u]);
+  }
+  float least = INFINITY;
+#pragma unroll
+  for (int u = 0; u < kSampleKeys; ++u) {
+#pragma unroll
+    for (int off = 16; off; off >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], off);
+    least = fminf(least, s[u]);
+  }
+  return least * rsqrtf(static_cast<float>(d)) - lse[t] < kPeakLog;
+}
+
 // Per (b, h, channel): {beta, 1/beta (0 at 0), c, mode}: 1 linear, 0 shifted, 2 wide.  The wide
 // channels of a head also go to its list (n_wide, then the channels), their dv zeroed for the key
-// pass to add to.
-__global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict__ v, const float *__restrict__ beta,
-                                                        int H, int T, int d, float4 *__restrict__ chan,
-                                                        int *__restrict__ wide, float *__restrict__ dv) {
+// pass to add to.  From kSampleT on one more block
+// samples the head's weights; a peaked one counts as kAllWide.
+constexpr int kAllWide = 1 << 20;
+__global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict__ q, const float *__restrict__ k,
+                                                        const float *__restrict__ v, const float *__restrict__ beta,
+                                                        const float *__restrict__ lse, int H, int T, int d, int causal,
+                                                        float4 *__restrict__ chan, int *__restrict__ wide,
+                                                        float *__restrict__ dv) {
+  if (blockIdx.y * 32 >= d) {
+    const size_t row0 = static_cast<size_t>(blockIdx.x) * T;
+    const bool peak = sample_peaked(q + row0 * d, k + row0 * d, lse + row0, T, d, causal);
+    if (__syncthreads_or(peak) && threadIdx.x == 0) atomicAdd(wide + static_cast<size_t>(blockIdx.x) * (d + 1), kAllWide);
+    return;
+  }
   __shared__ int s_wide[32];
   __shared__ float s_mx[32][33], s_mn[32][33], s_sm[32][33];
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, bh = blockIdx.x, j = blockIdx.y * 32 + lane;
@@ -87,7 +127,7 @@ __global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict_
                     !(lin || 0.5f * b * (mx - mn) + fmaxf(-logf(b), 0.f) <= kWideExp);
     if (wd) {
       int *list = wide + static_cast<size_t>(bh) * (d + 1);
-      list[1 + atomicAdd(list, 1)] = j;
+      list[1 + atomicAdd(list, 1) % kAllWide] = j;
     }
     s_wide[lane] = wd ? 1 : 0;
     chan[static_cast<size_t>(bh) * d + j] = make_float4(b, b > 0.f ? 1.f / b : 0.f, c, wd ? 2.f : (lin ? 1.f : 0.f));
@@ -250,7 +290,7 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
                    const float4 *__restrict__ chan, const int *__restrict__ wide, int *__restrict__ peaked,
                    float *__restrict__ power, float *__restrict__ head_power, float *__restrict__ dbp,
-                   float *__restrict__ dq, int T, int d, int causal) {
+                   float *__restrict__ dq, int T, int d, int causal, int wide_most) {
   using Lay = RowLay<DP>;
   constexpr int NC = DP / 16, CQ = DP / 4, kShare = kBT * CQ / 256;
   extern __shared__ __align__(16) float bwd_smem[];
@@ -260,12 +300,19 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
   const int rank = blockIdx.x, size = gridDim.x, bh = blockIdx.z;
   const int *wl = wide + static_cast<size_t>(bh) * (d + 1);
   const int n_wide = wl[0];
+  if (n_wide > wide_most) {  // pair by pair is faster, or needed
+    if (tid == 0) peaked[bh] = 1;
+    return;
+  }
   const int qt = static_cast<int>(gridDim.y) - 1 - static_cast<int>(blockIdx.y), t0 = qt * kBT;  // heaviest first
   const size_t base = static_cast<size_t>(bh) * T * d;
   const float4 *ch = chan + static_cast<size_t>(bh) * d;
   const bool vec = (d & 3) == 0;
   const float inv_sqrt_d = rsqrtf(static_cast<float>(d));
   if (tid < DP) sDb[tid] = 0.f;
+  // a pair with a weight below e^-60, here or (thread 0) in another CTA of the head: the head then goes
+  // pair by pair, and what the tiles give is dropped
+  bool peak = tid == 0 && *reinterpret_cast<volatile int *>(peaked + bh) != 0;
   {
     const int r = tid & 63, t = min(t0 + r, T - 1);
     const bool valid = t0 + r < T;
@@ -276,7 +323,8 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
       gm = fmaxf(fmaxf(gm, fmaxf(finite_abs(g4.x), finite_abs(g4.y))), fmaxf(finite_abs(g4.z), finite_abs(g4.w)));
     }
     sS[tid] = gm;
-    __syncthreads();
+    peak = __syncthreads_or(peak);
+    if (peak && size == 1) return;
     const float pw = row_power(fmaxf(fmaxf(sS[r], sS[kBT + r]), fmaxf(sS[2 * kBT + r], sS[3 * kBT + r]))), ipw = 1.f / pw;
     if (tid < kBT) {
       sS[4 * kBT + r] = pw;
@@ -332,11 +380,10 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int c = 0; c < NC; ++c) acc[i][c] = make_float2(0.f, 0.f);
-  bool peak = false;
   const int n_kt = causal ? qt + 1 : (T + kBT - 1) / kBT;
   for (int kt = rank; kt < n_kt; kt += size) {
     const int k0 = kt * kBT, nk = min(kBT, T - k0);
-    __syncthreads();  // the previous tile is consumed
+    if (__syncthreads_or(peak)) break;  // also: the previous tile is consumed
 #pragma unroll
     for (int u = 0; u < kShare; ++u) {
       const int e = tid + u * 256, r = e & 63, j = (e >> 6) * 4;
@@ -353,6 +400,7 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
       *reinterpret_cast<float4 *>(sKn + r * Lay::kNl + j) = k4;
     }
     __syncthreads();
+    const int others = tid == 0 ? *reinterpret_cast<volatile int *>(peaked + bh) : 0;  // lands under the contractions
     float2 s[2][4], U[2][4];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
@@ -382,6 +430,8 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
         ds[c][r] = vis ? expf(l) * (uv + R[r]) * pw[r] : 0.f;
       }
     }
+    if (peak) peaked[bh] = 1;
+    peak = peak || others != 0;
     for (int w = 0; w < n_wide; ++w) {
       const int j = wl[1 + w];
       const float b = ch[j].x, ib = ch[j].y;
@@ -414,7 +464,6 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
       }
     }
   }
-  if (peak) peaked[bh] = 1;
   float x[4 * NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c)
@@ -454,7 +503,7 @@ template <int DP>
 __global__ void __launch_bounds__(256, 1)
     bwd_key_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
-                   const float4 *__restrict__ chan, const int *__restrict__ wide, int *__restrict__ peaked,
+                   const float4 *__restrict__ chan, const int *__restrict__ wide, const int *__restrict__ peaked,
                    const float *__restrict__ power, const float *__restrict__ head_power, float *__restrict__ dbp,
                    float *__restrict__ dk, float *__restrict__ dv, int T, int d, int causal) {
   using Lay = KeyLay<DP>;
@@ -465,6 +514,7 @@ __global__ void __launch_bounds__(256, 1)
         *sS = bwd_smem + Lay::kS, *sR = bwd_smem + Lay::kR, *sDb = bwd_smem + Lay::kDb;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int rank = blockIdx.x, size = gridDim.x, bh = blockIdx.z, k0 = static_cast<int>(blockIdx.y) * kBT;
+  if (peaked[bh]) return;  // the head goes pair by pair
   const int *wl = wide + static_cast<size_t>(bh) * (d + 1);
   const int n_wide = wl[0];
   const size_t base = static_cast<size_t>(bh) * T * d;
@@ -489,7 +539,6 @@ __global__ void __launch_bounds__(256, 1)
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int c = 0; c < NC; ++c) ak[i][c] = ah[i][c] = a2h[i][c] = make_float2(0.f, 0.f);
-  bool peak = false;
   const int first = causal ? k0 / kRows : 0, n_rt = (T + kRows - 1) / kRows;
   for (int rt = first + rank; rt < n_rt; rt += size) {
     const int t0 = rt * kRows;
@@ -558,7 +607,6 @@ __global__ void __launch_bounds__(256, 1)
         const float sv = (r & 1) ? s[r >> 1][c].y : s[r >> 1][c].x, uv = (r & 1) ? U[r >> 1][c].y : U[r >> 1][c].x;
         const bool vis = i < T && t < T && (!causal || i <= t);
         const float l = fmaf(sv, inv_sqrt_d, -ls);
-        peak = peak || (vis && l < kPeakLog);
         lp[r][c] = vis ? l : -INFINITY;
         pv[c] = vis ? expf(l) : 0.f;
         ds[r][c] = vis ? pv[c] * (uv + Rt) * pw : 0.f;
@@ -611,7 +659,6 @@ __global__ void __launch_bounds__(256, 1)
       outer(a2h, p2, b);
     }
   }
-  if (peak) peaked[bh] = 1;
   float x[12 * NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c)
@@ -707,29 +754,35 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
         *head_power = reinterpret_cast<float *>(ws + w.head_power);
   int *wide = reinterpret_cast<int *>(ws + w.wide), *peaked = reinterpret_cast<int *>(ws + w.peaked);
   const int n_t = (T + kBT - 1) / kBT;
-  bwd_chan_kernel<<<dim3(BH, (d + 31) / 32), 1024, 0, stream>>>(v, beta, H, T, d, chan, wide, dv);
+  bwd_chan_kernel<<<dim3(BH, (d + 31) / 32 + (T >= kSampleT ? 1 : 0)), 1024, 0, stream>>>(q, k, v, beta, lse, H, T, d, causal, chan, wide, dv);
   // CTAs sharing a tile: until there are about four per SM, while each has a tile of the other side
   int size = 1;
   while (size < 8 && size * 2 <= n_t && static_cast<long long>(n_t) * BH * size < 3ll * num_sms) size *= 2;
+  // Wide channels beyond which a head goes pair by pair, where that is faster: 42 us each at B1 H4 T2048 d64
+  // against 2440 pair by pair, 2.4 against 75 at T64, 1.7 against 118 at B1 H1 T96 d128 (and the tiles' 62
+  // and 100 are spent besides where other heads stay).
+  const int wide_most = T < 256 ? 16 : 3 * d / 4;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = launch_cluster(bwd_row_kernel<DP>, dim3(size, n_t, BH), RowLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
                        static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, power, head_power, tile, dq, T, d,
-                       causal);
+                       causal, wide_most);
   if (e == cudaSuccess)
     e = launch_cluster(bwd_key_kernel<DP>, dim3(size, n_t, BH), KeyLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
-                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, static_cast<const float *>(power),
+                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), static_cast<const int *>(peaked), static_cast<const float *>(power),
                        static_cast<const float *>(head_power), tile, dk, dv, T, d, causal);
   return e;
 }
 
 }  // namespace
 
-// Pair by pair / tiled, us (both passes and the marks), causal: B*H = 4: d 64 T 32 61 / -, T 64 107 / 67,
-// T 256 402 / 75, T 2048 3563 / 468; d 128 T 64 94 / 103, T 96 135 / 106, T 2048 4141 / 819;
-// B*H = 64: d 16 T 64 78 / 56, T 1024 4452 / 770.  (A head with marked pairs runs both.)
+// Pair by pair / tiled, us, causal, plain heads: B*H = 1: d 16 T 64 64 / 46, d 64 T 64 62 / 63, T 80 76 / 67, T 300
+// 254 / 91, d 128 T 96 107 / 103, T 128 138 / 104; B*H = 4 T 2048 d 64 2440 / 478, d 128 4141 / 840; B*H = 384: d 64 T 64
+// 235 / 143, T 300 3420 / 1096, d 128 T 96 740 / 592; B*H = 64 d 16 T 1024 4452 / 770.
 bool bwd_tile_takes(int B, int H, int T, int d) {
-  return d <= 128 && T >= (d <= 64 ? 64 : 96) && static_cast<long long>(T) <= 64ll * 65535 && static_cast<long long>(B) * H <= 65535;
+  const bool few = static_cast<long long>(B) * H * T <= kBwdFewRows;
+  const int least = d <= 32 ? 64 : d <= 64 ? (few ? 80 : 64) : (few ? 128 : 96);
+  return d <= 128 && T >= least && static_cast<long long>(T) <= 64ll * 65535 && static_cast<long long>(B) * H <= 65535;
 }
 
 size_t bwd_workspace_bytes(int B, int H, int T, int d) {

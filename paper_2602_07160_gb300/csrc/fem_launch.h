@@ -167,6 +167,9 @@ cudaError_t launch_bwd_f32(const float *q, const float *k, const float *v, const
 cudaError_t launch_bwd_tile(const float *q, const float *k, const float *v, const float *beta, const float *out,
                             const float *lse, const float *dout, float *dq, float *dk, float *dv, float *dbeta, int B,
                             int H, int T, int d, int causal, void *ws, int num_sms, cudaStream_t stream);
+// Rows up to which the gradients' pair-by-pair kernels take one to a warp at 33 to 64 channels, half as many at
+// other widths (launch_bwd_pairs has the figures).
+constexpr long long kBwdFewRows = 8192;
 // Pair by pair; with peaked ([B H] marks) only the heads marked, their dbeta sums added to dbeta
 // [B H, d] instead of [H, d].
 cudaError_t launch_bwd_pairs(const float *q, const float *k, const float *v, const float *beta, const float *out,
