@@ -54,6 +54,8 @@
 // then barriers and per-channel state.  Every mbarrier completes once per use
 // of what it guards, and no waiter can fall two phases behind: a buffer's
 // next use always waits for the previous one.
+#include <algorithm>
+
 #include "fem_common.cuh"
 #include "fem_launch.h"
 #include "fem_order.h"
@@ -896,6 +898,26 @@ static cudaError_t launch_tc_d(const CUtensorMap &tq, const CUtensorMap &tk, con
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The d = 64 read's form: two CTAs per SM (fem_tc_half.cu, true) or one (this file).  With a CTA to itself on
+// every SM one is faster, and so it is where a causal grid's heaviest CTAs set the time; with the SMs full, or
+// few key tiles a CTA, two.  Between those the longer of the grid's work over its slots and the last head
+// group's heaviest CTA behind the groups before it decides: a CTA takes a fixed time (one per SM 7.4 us, two 8)
+// and per key tile 0.62 or, alone at the end, 0.76 us; two 1.3 and 1.05.  Whole calls, one / two per SM, us:
+// causal B1 H12 T1024 (96 CTAs) 43 / 47, H5 T4096 (160) 58 / 69, H16 T2048 (256) 54 / 58, H4 T8192 (256) 80 /
+// 109, H10 T8192 (640) 174 / 192; H50 T512 (200) 46 / 42, H20 T2048 (320) 64 / 60, H16 T8192 (1024) 235 / 215,
+// B8 H12 T2048 (1536) 185 / 164; full H10 T2048 (160) 54 / 49, B64 H6 T197 (768) 56 / 43.
+static bool two_per_sm(int BH, int n_qt, int causal, int num_sms) {
+  const double ctas = static_cast<double>(n_qt) * BH;
+  if (ctas <= num_sms) return false;
+  if (!causal || n_qt <= 6) return true;
+  const int before = (BH - 1) / kHeadGroup * kHeadGroup;  // heads of the groups before the last
+  auto us = [&](double tile, double lone, double fixed, int slots) {
+    const double head = (0.5 * n_qt * (n_qt + 1.0) * tile + n_qt * fixed) / slots;
+    return std::max(BH * head, before * head + n_qt * lone + fixed);
+  };
+  return us(1.3, 1.05, 8.0, 2 * num_sms) < us(0.62, 0.76, 7.4, num_sms);
+}
+
 cudaError_t launch_tc(int d, const CUtensorMap &tq, const CUtensorMap &tk, const CUtensorMap &te,
                       const CUtensorMap *te0, float *out, const float *beta, const BankWorkspace &w, float *lse,
                       int BH, int H, int T, int causal, const TcGate *gate, unsigned *err, int num_sms,
@@ -909,12 +931,7 @@ cudaError_t launch_tc(int d, const CUtensorMap &tq, const CUtensorMap &tk, const
       return launch_tc_d<128, true>(tq, tk, te, *te0, out, beta, w, lse, BH, H, T, causal, *gate, err, stream, pdl);
     return cudaErrorInvalidValue;
   }
-  // d = 64: two CTAs per SM (fem_tc_half.cu) once the grid holds more than one CTA per SM; with a CTA
-  // to itself on every SM this file's form is faster.  One / two per SM, us: B1 H1 T2048 causal (16 CTAs)
-  // 20.1 / 26.1, B1 H12 T1024 (96) 18.0 / 22.0, B1 H4 T4096 (128) 32.2 / 42.5, B8 H12 T512 (384) 31.4 /
-  // 29.3, B64 H6 T197 full (768) 43.6 / 29.3, B8 H12 T2048 (1536) 130.8 / 112.6.
-  const long long ctas = static_cast<long long>((T + kBlockQ - 1) / kBlockQ) * BH;
-  if (d == 64 && ctas > num_sms)
+  if (d == 64 && two_per_sm(BH, (T + kBlockQ - 1) / kBlockQ, causal, num_sms))
     return launch_tc_half(tq, tk, te, out, beta, w, lse, BH, H, T, causal, err, stream, pdl);
   if (d == 64)
     return launch_tc_d<64, false>(tq, tk, te, te, out, beta, w, lse, BH, H, T, causal, none, err, stream, pdl);
