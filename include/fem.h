@@ -205,7 +205,9 @@ int fem_decode(const void *q, const void *k, const void *v, const float *beta, f
  * In chunks of 64 steps, in fp32 on CUDA cores: each chunk's own state, the start
  * states by a scan over chunks, then the outputs (one launch for T <= 64).
  * Allocates its workspace (a state per chunk; at most 256 MB, heads and runs of
- * chunks taken in turn beyond) stream-ordered on `stream`.
+ * chunks taken in turn beyond) stream-ordered on `stream`, from a pool of its own
+ * with fem_gla_fwd_tc that keeps up to 320 MB per device once they have used them
+ * and returns what is beyond at the next synchronisation.
  */
 int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *logdecay,
                 const float *beta, float *out, float *logz, int B, int H, int T, int m, int d,
@@ -220,7 +222,8 @@ int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *l
  * (tcgen05); the state itself is kept in fp32.  Up to T = 256 a pair of CTAs
  * per (b, h) walks the chunks; beyond, the chunks run in parallel around a scan
  * of their states, with a workspace (at most 320 MB, or one head's 66 KB a
- * chunk) allocated stream-ordered on `stream`.  Channels
+ * chunk) allocated like fem_gla_fwd's (where there is no room for it the pair of
+ * CTAs walks).  Channels
  * with beta < 1/4 use the bank expm1(beta (v - c)) / beta anchored at the
  * mean of the values so far, the others exp(beta v - lambda) with a log-scaled
  * state.  Accuracy is the bf16 read's for values of unit spread (max abs 2e-2,

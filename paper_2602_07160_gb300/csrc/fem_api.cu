@@ -37,6 +37,7 @@ struct DeviceState {
   // stream-ordered workspaces come from this pool, which keeps freed memory for
   // the next call instead of returning it to the driver at every synchronisation
   cudaMemPool_t pool = nullptr;
+  cudaMemPool_t scan_pool = nullptr;  // the GLA reads', which keeps kScanKeep at most
   unsigned *beta_bad = nullptr;
   // copy streams of fem_fwd_host, created on its first call
   cudaStream_t copy_in = nullptr, copy_out = nullptr;
@@ -124,13 +125,19 @@ int debug_check_beta_host(const float *beta, long long n) {
   return FEM_OK;
 }
 
-// Stream-ordered workspace from the device's library pool (free with
-// cudaFreeAsync).  The pool is created by the first entry point that
-// allocates on the device.
-cudaError_t ws_alloc(DeviceState *ds, void **p, size_t bytes, cudaStream_t s) {
+// Stream-ordered workspace from one of the device's library pools (free with
+// cudaFreeAsync): ds->pool, or with `scan` ds->scan_pool, which keeps kScanKeep at most; what
+// is freed beyond goes back to the device at the next synchronisation.  That holds the GLA reads'
+// largest group of heads, so a run of such calls allocates once (with nothing kept a call at B4 H16
+// T8192 that is waited for takes 965 us instead of 377).  A pool is created by the first entry
+// point that allocates from it.
+constexpr uint64_t kScanKeep = uint64_t(320) << 20;
+
+cudaError_t ws_alloc(DeviceState *ds, void **p, size_t bytes, cudaStream_t s, bool scan = false) {
+  cudaMemPool_t &slot = scan ? ds->scan_pool : ds->pool;
   {
     std::lock_guard<std::mutex> lock(g_mutex);
-    if (!ds->pool) {
+    if (!slot) {
       int dev = 0;
       cudaError_t e = cudaGetDevice(&dev);
       if (e != cudaSuccess) return e;
@@ -143,24 +150,24 @@ cudaError_t ws_alloc(DeviceState *ds, void **p, size_t bytes, cudaStream_t s) {
       cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
       if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
       e = cudaMemPoolCreate(&pool, &props);
-      uint64_t keep = ~uint64_t(0);
+      uint64_t keep = scan ? kScanKeep : ~uint64_t(0);
       if (e == cudaSuccess && (e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess)
         cudaMemPoolDestroy(pool);
       const cudaError_t back = cudaThreadExchangeStreamCaptureMode(&mode);
       if (e != cudaSuccess) return e;
-      ds->pool = pool;
+      slot = pool;
       if (back != cudaSuccess) return back;
     }
   }
-  return cudaMallocFromPoolAsync(p, bytes, ds->pool, s);
+  return cudaMallocFromPoolAsync(p, bytes, slot, s);
 }
 
 // The same for a caller that has a form without a workspace: none (nullptr) for 0 bytes or where
 // there is no room, which is slower but not refused.
-cudaError_t ws_alloc_if(DeviceState *ds, void **p, size_t bytes, cudaStream_t s) {
+cudaError_t ws_alloc_if(DeviceState *ds, void **p, size_t bytes, cudaStream_t s, bool scan = false) {
   *p = nullptr;
   if (!bytes) return cudaSuccess;
-  const cudaError_t e = ws_alloc(ds, p, bytes, s);
+  const cudaError_t e = ws_alloc(ds, p, bytes, s, scan);
   if (e != cudaErrorMemoryAllocation) return e;
   cudaGetLastError();
   *p = nullptr;
@@ -548,7 +555,7 @@ int fem_gla_fwd_tc(const float *qf, const float *kf, const float *v, const float
     return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   void *ws = nullptr;
-  cudaError_t e = ws_alloc_if(ds, &ws, gla_par_workspace_bytes(B * H, T), s);
+  cudaError_t e = ws_alloc_if(ds, &ws, gla_par_workspace_bytes(B * H, T), s, true);
   if (e != cudaSuccess) return map_cuda(e);
   rc = map_cuda(launch_gla_tc(qf, kf, v, logdecay, beta, out, logz, B, H, T, ws, ds->err, s));
   if (!ws) return rc;
@@ -578,11 +585,11 @@ int fem_gla_fwd(const float *qf, const float *kf, const float *v, const float *l
   void *ws = nullptr;
   size_t cap = size_t(256) << 20;
   size_t bytes = gla_workspace_bytes(B * H, T, m, d, cap);
-  cudaError_t e = ws_alloc_if(ds, &ws, bytes, s);
+  cudaError_t e = ws_alloc_if(ds, &ws, bytes, s, true);
   if (e == cudaSuccess && bytes && !ws) {  // little room: short runs of chunks
     cap = size_t(1) << 20;
     bytes = gla_workspace_bytes(B * H, T, m, d, cap);
-    e = ws_alloc(ds, &ws, bytes, s);
+    e = ws_alloc(ds, &ws, bytes, s, true);
   }
   if (e != cudaSuccess) return map_cuda(e);
   rc = map_cuda(launch_gla(qf, kf, v, logdecay, beta, out, logz, B * H, H, T, m, d, cap, ws, s));
