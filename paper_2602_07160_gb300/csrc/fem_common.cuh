@@ -260,6 +260,11 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, uns
 // mean, beta spread^2 / 2 away), where 1 / beta can be infinite and beta v has few bits.
 __device__ __forceinline__ float normal_beta(float b) { return fabsf(b) < 0x1p-126f ? 0.f : b; }
 
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t *>(&v);
+}
+
 __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   const __half2 v = __floats2half2_rn(lo, hi);
   return *reinterpret_cast<const uint32_t *>(&v);

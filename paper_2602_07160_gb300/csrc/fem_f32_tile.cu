@@ -599,8 +599,8 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
             again |= 1u << (4 * c + r);
         }
         if (b > 0.f) {
-          // log1p(b x) or log(x), the latter as n ln 2 + log(mantissa) in two parts, over b and onto c
-          // with the rounding errors of both steps carried: |c - o| may be several times |o|
+          // log1p(b x) or log(x), the latter as n ln 2 + log(mantissa) with ln 2 in two parts (Cody and Waite),
+          // over b and onto c with the rounding errors of both steps carried: |c - o| may be several times |o|
           float hi, lo = 0.f;
           if (lin) {
             hi = log1pf(b * x);

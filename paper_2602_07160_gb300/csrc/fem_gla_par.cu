@@ -44,8 +44,7 @@
 //
 // B4 H16 T8192: 23 + 10 + 102 + 34 + 171 us, 356 in all (the inputs and outputs once are 80).
 // local and scan run at 4.7 and 4 TB/s; out is bound by its phases' latencies (2 us of loads, then scores,
-// mask, sums and read behind one another, two chunks an SM at a time: TMEM holds no more);
-//
+// mask, sums and read behind one another, two chunks an SM at a time: TMEM holds no more).  All five run
 // over groups of heads (gla_par_group).
 //
 // The bf16 operands' relative error (2^-9) reaches o as about 2^-9 |v - c| (linear)
@@ -56,17 +55,15 @@
 // range could then carry it) the entry is recomputed exactly, from the scores of
 // the bf16 operands in fp32, with the running maximum of the row's visible keys as the shift.
 #include "fem_common.cuh"
+#include "fem_gla_tc.cuh"
 #include "fem_launch.h"
 
 namespace fem {
 namespace {
 
-constexpr int kGC = 128;   // steps per chunk (rows of S, TMEM lanes)
-constexpr int kGM = 64;    // feature width
 constexpr int kGD = 64;    // value channels
 constexpr int kGN = 80;    // U's columns: the channels, the constant one, zero padding to a multiple of 16
 constexpr int kSt = (kGD + 1) * kGM;  // floats of a state: channel rows of 64 features, Z's last
-constexpr float kGlaLinBeta = 0.25f;
 constexpr uint32_t kImg = 16384;  // a 128 x 64 bf16 operand image
 
 // Workspace of a group of heads; per (head, chunk) unless noted.
@@ -82,36 +79,8 @@ struct GlaTcWs {
   float *s;       // [65][64]
 };
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&v);
-}
 __device__ __forceinline__ float2 unpack_bf16x2(uint32_t w) {
   return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
-// expm1(y) / beta for y = beta x: x times the series of expm1(y) / y for |y| < 1/2
-// (truncation below 4e-6 relative), (e^y - 1) / beta beyond (ex2.approx: the result
-// is rounded to bf16); x itself at beta = 0.
-__device__ __forceinline__ float em1_beta_fast(float x, float y, float rb) {
-  float p = fmaf(y, 1.f / 720.f, 1.f / 120.f);  // both forms, then a select: no branch per element
-  p = fmaf(y, p, 1.f / 24.f);
-  p = fmaf(y, p, 1.f / 6.f);
-  p = fmaf(y, p, 0.5f);
-  p = fmaf(y, p, 1.f);
-  const float far = (__expf(y) - 1.f) * rb;
-  return fabsf(y) < 0.5f ? x * p : far;
-}
-
-// log1p(x) for x > -1: the series to x^5 for |x| < 2^-6 (truncation below 2^-36
-// relative), lg2.approx of 1 + x beyond.
-__device__ __forceinline__ float log1p_fast(float x) {
-  float p = fmaf(x, 0.2f, -0.25f);  // both forms, then a select
-  p = fmaf(x, p, 1.f / 3.f);
-  p = fmaf(x, p, -0.5f);
-  p = fmaf(x, p, 1.f);
-  const float far = __logf(1.f + x);
-  return fabsf(x) < 0.015625f ? x * p : far;
 }
 
 // 8 consecutive fp32 as bf16 into a 16-byte chunk of a 128-byte-swizzled row.
@@ -765,7 +734,7 @@ size_t gla_par_layout(int heads, int n_ch, uint8_t *p, GlaTcWs *w) {
 
 // Heads per group: as many as keep the group's workspace below 320 MB (4.3 MB a head at T = 8192), at
 // least one; groups of equal size.  Fewer launches and fuller waves outweigh what smaller groups keep in
-// L2: 64 heads of T = 8192 in groups of 9, 16, 32 or all: 851, 637, 557, 512 us.
+// L2: 64 heads of T = 8192 in groups of 13, 22 or all: 452, 412, 348 us.
 int gla_par_group(int BH, int n_ch) {
   const size_t fit = (size_t{320} << 20) / gla_par_layout(1, n_ch, nullptr, nullptr);
   const size_t cap = fit < 1 ? 1 : (fit > 16384 ? 16384 : fit);

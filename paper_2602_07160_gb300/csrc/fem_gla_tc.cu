@@ -43,19 +43,17 @@
 // recomputed exactly from the fp32 scores and the values, with the running
 // maximum of the row's visible keys as the shift.
 #include "fem_common.cuh"
+#include "fem_gla_tc.cuh"
 #include "fem_launch.h"
 
 namespace fem {
 namespace {
 
-constexpr int kGC = 128;        // steps per chunk (rows of S, TMEM lanes)
-constexpr int kGM = 64;         // feature width
 constexpr int kVD = 64;         // value channels of a head (the row width of v and out)
 constexpr int kGD = 32;         // value channels of a CTA: two CTAs share a head
 constexpr int kGN = 48;         // the CTA's channels, the constant channel, zero padding to a multiple of 16
 constexpr int kQtr = 256 / kGD;  // groups of keys in the per-channel passes (thread = channel and group)
 constexpr int kKg = kGC / kQtr;  // keys per group
-constexpr float kGlaLinBeta = 0.25f;
 
 struct GLay {
   static constexpr uint32_t kQ32 = 0, kK32 = 32768, kV32 = 65536;  // the chunk's fp32 inputs
@@ -84,35 +82,6 @@ struct GLay {
 // TMEM columns (32-column aligned): S in fp32 (kept for the exact rows), the masked bf16 A,
 // the three accumulators
 constexpr uint32_t kColS = 0, kColA = 128, kColInter = 192, kColIntra = 288, kColU = 384;
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&v);
-}
-
-// expm1(y) / beta for y = beta x: x times the series of expm1(y) / y for |y| < 1/2
-// (truncation below 4e-6 relative), (e^y - 1) / beta beyond (ex2.approx: the result
-// is rounded to bf16); x itself at beta = 0.
-__device__ __forceinline__ float em1_beta_fast(float x, float y, float rb) {
-  float p = fmaf(y, 1.f / 720.f, 1.f / 120.f);  // both forms, then a select: no branch per element
-  p = fmaf(y, p, 1.f / 24.f);
-  p = fmaf(y, p, 1.f / 6.f);
-  p = fmaf(y, p, 0.5f);
-  p = fmaf(y, p, 1.f);
-  const float far = (__expf(y) - 1.f) * rb;
-  return fabsf(y) < 0.5f ? x * p : far;
-}
-
-// log1p(x) for x > -1: the series to x^5 for |x| < 2^-6 (truncation below 2^-36
-// relative), lg2.approx of 1 + x beyond.
-__device__ __forceinline__ float log1p_fast(float x) {
-  float p = fmaf(x, 0.2f, -0.25f);  // both forms, then a select
-  p = fmaf(x, p, 1.f / 3.f);
-  p = fmaf(x, p, -0.5f);
-  p = fmaf(x, p, 1.f);
-  const float far = __logf(1.f + x);
-  return fabsf(x) < 0.015625f ? x * p : far;
-}
 
 // 8 consecutive fp32 as bf16 into a 16-byte chunk of a 128-byte-swizzled row.
 __device__ __forceinline__ void st_bf16x8(uint8_t *dst, const float *src, float scale) {

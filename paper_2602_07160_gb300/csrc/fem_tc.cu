@@ -129,11 +129,6 @@ enum : int {
   kBarSide = 33      // + side slot (8): tile k's rescale factors and moved-channel mask are in shared memory
 };
 
-__device__ __forceinline__ uint32_t pack_bf162(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t *>(&v);
-}
-
 // ATTN: the attention-mode comparator -- plain softmax attention
 // o = sum_i p_t(i) v_i, the same kernel with V itself (bf16) as the second
 // operand and P in bf16: no value bank, no shifts, no guard.
@@ -417,7 +412,7 @@ __global__ void __launch_bounds__(384, 1)
             const float2 x = __ffma2_rn(make_float2(s[c * 32 + 2 * i], s[c * 32 + 2 * i + 1]), scale2, negm2);
             const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));
             ls[i & 3] = __fadd2_rn(ls[i & 3], e);
-            p[i] = ATTN ? pack_bf162(e.x, e.y) : pack_half2(e.x, e.y);
+            p[i] = ATTN ? pack_bf16x2(e.x, e.y) : pack_half2(e.x, e.y);
           }
           tmem_st16(tS + c * 16, p);
         }

@@ -1,6 +1,6 @@
 // Tensor-core read at d = 64 with two CTAs per SM (sm_103a, tcgen05): the read
 // of fem_tc.cu (same operands, softmax, rescale, guard and entry list, the same
-// results bit for bit) in a CTA of half an SM's tensor memory, shared memory and
+// results up to the order of a rescale's two factors) in a CTA of half an SM's tensor memory, shared memory and
 // registers.
 //
 // What bounded the one-CTA form: a CTA holds the SM while it fills its pipeline
@@ -86,16 +86,15 @@ struct HalfLayout {
 enum : int {
   kHQ = 0,
   kHKFull = 1,    // + stage (2)
-  kHKEmpty = 3,   // + stage (2)
-  kHEFull = 5,    // + slot (3)
-  kHEEmpty = 8,   // + slot (3)
-  kHSide = 11,    // + slot (4)
-  kHSFull = 15,   // S_k complete
-  kHSFree = 16,   // the softmax has read S_k (128 arrivals)
-  kHPFull = 17,   // P_k written and acc rescaled (128 arrivals)
-  kHPvDone = 18,  // P_k E_k complete
-  kHAll = 19,     // everything the two issuers started is complete (2 arrivals)
-  kHCount = 20
+  kHEFull = 3,    // + slot (3)
+  kHEEmpty = 6,   // + slot (3)
+  kHSide = 9,     // + slot (4)
+  kHSFull = 13,   // S_k complete
+  kHSFree = 14,   // the softmax has read S_k (128 arrivals)
+  kHPFull = 15,   // P_k written and acc rescaled (128 arrivals)
+  kHPvDone = 16,  // P_k E_k complete
+  kHAll = 17,     // everything the two issuers started is complete (2 arrivals)
+  kHCount = 18
 };
 
 __global__ void __launch_bounds__(192, 2)
