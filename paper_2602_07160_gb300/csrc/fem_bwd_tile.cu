@@ -20,7 +20,7 @@
 // [1, 2) there), which comes back at dS; the sums over rows take p times the row's
 // power over the head's largest, which comes back at dv and dbeta.  So nothing depends
 // on the scale of g, and what fp32's range drops from p e^b (2^-150) stays, times e^a,
-// below 2^-46 of the head's largest cotangent.
+// below 2^-40 of the head's largest cotangent.
 // All exponents carry their rounding errors (exp_tilt), which keeps the gradients'
 // error at that of exp(x) taken directly.  Channels whose spread exceeds that (or is
 // not finite) take no part in the contractions; their terms are formed pair by pair
@@ -48,7 +48,7 @@ namespace {
 
 constexpr int kBT = 64;           // rows and keys of a tile (rows of the other side: kRows below)
 constexpr int kBLd = 68;          // leading dimension of a transposed 64-row tile
-constexpr float kWideExp = 72.f;  // largest |a|, |b| of a factored channel: 2^+-104
+constexpr float kWideExp = 76.f;  // largest |a|, |b| of a factored channel: 2^+-110
 constexpr float kPeakLog = -60.f;
 
 // A head's sample of pairs for the mark of peaked priors: warp w takes row T - 1 - w T / 32 and 16 of its keys,
