@@ -159,7 +159,7 @@ __device__ __forceinline__ float4 bank_coef(bool lin, float b, float c) {
 // ---------------------------------------------------------------------------
 // A read's plan and bank; beta null is beta = 0 (the prior mean).  The gated read makes two of the same
 // V, as grid z = 0 and 1 here and as alternate tasks of the bank kernel (two plans and two banks in turn,
-// each 7 to 8 us at B4 H4 T2048 d128 and far from filling the chip, made that call 118 us; it is 106 now).
+// each 7 to 8 us at B4 H4 T2048 d128 and far from filling the chip: that call 116.6 us, 106.4 as one each).
 struct BankSet {
   const float *beta;
   ChanInfo *chan;
@@ -490,8 +490,8 @@ __global__ void __launch_bounds__(256, 2) bank_kernel(const __grid_constant__ CU
 // group) of the key tiles w / 4 and, with more than two (TP = 2), w / 4 + 2; its
 // rows stay in registers from the statistics to the bank, so V is read once, and
 // those of one or two tiles leave room for four or three blocks per SM (with the rows of four
-// tiles at a time, V read again for the bank and two blocks per SM, a call at B64 H6 T197 d64 took 47.5 us
-// and takes 43.2; B32 H8 T256 d128 162 -> 152, B64 H16 T512 d128 841 -> 810).
+// tiles at a time, V read again for the bank and two blocks per SM, a full-prior call at B64 H6 T197 d64 took
+// 46.8 us and takes 42.8; B32 H8 T256 d128 64.7 -> 55.9, B64 H16 T512 d128 422 -> 391).
 // Lane l takes rows l, l + 32, l + 64, l + 96 of a tile, so a channel's bank
 // form is uniform across the warp and all eight warps work on sequences of two
 // key tiles.  A warp load touches 32 row segments,

@@ -319,7 +319,7 @@ __device__ __forceinline__ float dec_read(float b, float L, float c, float A, fl
 // there are more than n, r + n (both in flight from the start); the CTAs' partials meet in shared
 // memory instead of a workspace and a second launch.  What bounds it is the latency of a chunk and of
 // the calls in front of it: B1 H12 T1000 d64 5.7 us in a graph against 6.8 for the two launches, and
-// a call from the host 15.2 against 19.7 (no workspace, one launch).
+// a call from the host is one launch and a workspace shorter.
 constexpr int kDecCtas = 8, kDecOwn = 2;  // CTAs of a cluster (portable), chunks of a CTA at most
 
 template <int D>
