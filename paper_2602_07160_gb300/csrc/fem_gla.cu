@@ -30,8 +30,8 @@
 // beta v + gamma_last - gamma_i, and a state's log-scale mu the largest of its terms', decaying with
 // the prior; the normaliser's is 0.  lam may belong to a key that a row does not see: where in_t is
 // below 2^-90 of the row's in-chunk mass, or both parts together of the row's whole mass (fp32's
-// range could then hide terms that count), or not finite, the entry is read again key by key, from
-// the keys the row sees and the start state.  The decay's sums are taken in float64 and kept as
+// range could then hide terms that count), or not finite, the entry is read again around the largest term
+// of the keys the row sees, with the start state (read_again, read_rows).  The decay's sums are taken in float64 and kept as
 // two floats, so a difference costs the rounding of its own size (steps of -60 are exact to 1e-7);
 // steps below kGlaFloor count as it: their weights are zero either way.
 //
@@ -40,7 +40,7 @@
 // 123 in all, against 331 for a scan that walked segments of the sequence step by step, four lanes to a
 // channel's state (passes of 90 and 229 us, one dependent step at a time); B1 H1 T64 25 against 122,
 // B4 H16 T512 m16 d32 62 against 79.  Values of ten times unit spread with beta up to 100 send most
-// entries to the key-by-key read: 510 us at the first size.
+// entries to read_again: 354 us at the first size, 406 for the scan.
 #include "fem_common.cuh"
 #include "fem_f32.cuh"
 #include "fem_launch.h"
@@ -53,6 +53,7 @@ constexpr int kThreads = 256;         // thread (ty, tx): four rows (or features
 constexpr int kLd = kSteps + 4;       // leading dimension of the transposed Q and K tiles
 constexpr float kGlaGuard = 0x1p-90f;
 constexpr float kGlaFloor = -1e6f;
+constexpr int kFewFlagged = 24;  // threads of a block with flagged entries up to which rows are read one by one
 constexpr float kGlaSmallBeta = 0x1p-5f, kGlaSmallTilt = 0.25f;
 
 // Workspace of a group of heads and a run of chunks; per (head, chunk) unless noted.
@@ -318,13 +319,246 @@ struct OutF32 {
   static constexpr int kFloats = kS + kSteps * kSteps;
 };
 
+// The read of one entry from its in-chunk sum acc at the shift m (linear: acc alone) and the state's part.
+__device__ __forceinline__ float read_entry(float b, float m, float acc, float ix, float mu, float et, float gt, float den,
+                                            bool state) {
+  if (!(b > 0.f)) return lin_read(b, (state ? fmaf(et, ix, acc) : acc) / den);
+  const float la = acc == 0.f ? -INFINITY : m + logf(acc);
+  const float lb = ix == 0.f ? -INFINITY : mu + gt + logf(ix);
+  const float hi = fmaxf(la, lb), lo = fminf(la, lb);
+  const float ln = hi == -INFINITY ? hi : hi + log1pf(expf(lo - hi));
+  return ((la != la ? la : lb != lb ? lb : ln) - logf(den)) / b;
+}
+
+// The block's flagged entries (s_flag: 64 bits a row) once more, from the keys their rows see and the start
+// state: the scores again, then in the warps that have any the largest beta v + decay of the visible keys and
+// the sum around it, four rows against four channels a thread as in the sums before.  B4 H4 T2048 m64 d128 with
+// values of 10, 30 and 100 times unit spread and beta up to 100, 100 and 200: 354, 354 and 352 us a call; with
+// read_rows alone 577, 673, 763.
+template <int M>
+__device__ __noinline__ void read_again(float *smem, const float2 *gam, const float *s_den, const float *s_b,
+                                        const unsigned (*s_flag)[2], const float *v, float *out, int h0, int T, int d,
+                                        int dp, int c0, int nb, int vec, const GlaWs &w) {
+  using Lay = OutF32<M>;
+  // (the block's place again from the launch's parameters: handed over, it stays in registers through the read)
+  const int hd = blockIdx.z, j0 = blockIdx.y * kCh, c = c0 + blockIdx.x, rows = min(kSteps, T - c * kSteps);
+  const size_t r0 = static_cast<size_t>(h0 + hd) * T + static_cast<size_t>(c) * kSteps;
+  const size_t task = static_cast<size_t>(hd) * nb + blockIdx.x;
+  const bool state = c > 0;
+  v += r0 * d;
+  out += r0 * d;
+  const float *sQ = smem + Lay::kQ, *sK = smem + Lay::kK;
+  float *sV = smem + Lay::kE, *sS = smem + Lay::kS;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, jq = j0 + tx * 4;
+  const float4 b = ld4(s_b + tx * 4);
+  unsigned flags = 0;  // bit 4 r + q is row 4 ty + r, channel 4 tx + q
+#pragma unroll
+  for (int r = 0; r < 4; ++r) flags |= ((s_flag[ty * 4 + r][tx >> 3] >> ((tx & 7) * 4)) & 15u) << (4 * r);
+  {
+    float4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = ty + 16 * u;
+      x[u] = r < rows ? ld_row4(v + static_cast<size_t>(r) * d, jq, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    lin_values(b, x);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) *reinterpret_cast<float4 *>(sV + (ty + 16 * u) * kCh + tx * 4) = x[u];
+    float s[4][4];  // [key][row]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) s[i][r] = 0.f;
+#pragma unroll 4
+    for (int f = 0; f < M; ++f) {
+      const float4 q4 = ld4(sQ + f * kLd + ty * 4), k4 = ld4(sK + f * kLd + tx * 4);
+      const float qr[4] = {q4.x, q4.y, q4.z, q4.w}, kr[4] = {k4.x, k4.y, k4.z, k4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[i][r] = fmaf(qr[r], kr[i], s[i][r]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      *reinterpret_cast<float4 *>(sS + (tx * 4 + i) * kSteps + ((ty ^ tx) << 2)) = make_float4(s[i][0], s[i][1], s[i][2], s[i][3]);
+  }
+  __syncthreads();
+  if (!__any_sync(0xffffffffu, flags != 0u)) return;
+  // exponents in units of ln 2; a linear channel's terms are its values times the decays
+  const float bj[4] = {b.x, b.y, b.z, b.w};
+  float b2[4], m[4][4], acc[4][4];
+  float2 g[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    g[r] = gam[ty * 4 + r];
+    b2[r] = bj[r] > 0.f ? bj[r] * kLog2e : 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      m[r][q] = -INFINITY;
+      acc[r][q] = 0.f;
+    }
+  }
+  const int last = min(rows, (tid >> 5) * 8 + 8);  // a warp's rows see no key from here on
+  for (int i = 0; i < last; ++i) {
+    const float4 x4 = ld4(sV + i * kCh + tx * 4);
+    const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+    const float2 gi = gam[i];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float dg = i <= ty * 4 + r ? sum_diff(g[r], gi) * kLog2e : -INFINITY;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float y = fmaf(b2[q], x[q], dg);
+        m[r][q] = fmaxf(m[r][q], i <= ty * 4 + r ? y : -INFINITY);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (!(bj[q] > 0.f) || m[r][q] == -INFINITY) m[r][q] = 0.f;
+  for (int i = 0; i < last; ++i) {
+    const float4 x4 = ld4(sV + i * kCh + tx * 4), s4 = ld4(sS + i * kSteps + ((ty ^ (i >> 2)) << 2));
+    const float x[4] = {x4.x, x4.y, x4.z, x4.w}, sc[4] = {s4.x, s4.y, s4.z, s4.w};
+    const float2 gi = gam[i];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (i > ty * 4 + r) continue;
+      const float dg = sum_diff(g[r], gi) * kLog2e;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float y = b2[q] > 0.f ? fmaf(b2[q], x[q], dg) : dg, e = ex2_approx(y - m[r][q]);
+        acc[r][q] = fmaf(b2[q] > 0.f ? sc[r] : sc[r] * x[q], e, acc[r][q]);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int t = ty * 4 + r;
+    const float e0 = expf(g[r].x), et = fmaf(e0, g[r].y, e0), gt = g[r].x + g[r].y;
+    float ix[4] = {0.f, 0.f, 0.f, 0.f};
+    if (state && ((flags >> (4 * r)) & 15u)) {
+#pragma unroll 8
+      for (int f = 0; f < M; ++f) {
+        const float qr = sQ[f * kLd + t];
+        const float4 u4 = ld4(w.u + (task * M + f) * dp + jq);
+        ix[0] = fmaf(qr, u4.x, ix[0]);
+        ix[1] = fmaf(qr, u4.y, ix[1]);
+        ix[2] = fmaf(qr, u4.z, ix[2]);
+        ix[3] = fmaf(qr, u4.w, ix[3]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (!((flags >> (4 * r + q)) & 1u)) continue;
+      const float mu = state && bj[q] > 0.f ? w.mu[task * dp + jq + q] : 0.f;
+      out[static_cast<size_t>(t) * d + jq + q] =
+          read_entry(bj[q], m[r][q] * kLn2, acc[r][q], ix[q], mu, et, gt, s_den[t], state);
+    }
+  }
+}
+
+// The same for few flagged entries: a warp per row, its lanes over channels or keys (at kFewFlagged 24 or 40 a
+// call at 3 times unit spread 235 or 227 us, at 10 times 333 or 360).
+template <int M>
+__device__ __noinline__ void read_rows(float *smem, const float2 *gam, const float *s_den, const float *s_b,
+                                       const unsigned (*s_flag)[2], const float *v, float *out, int h0, int T, int d,
+                                       int dp, int c0, int nb, const GlaWs &w) {
+  using Lay = OutF32<M>;
+  const int hd = blockIdx.z, j0 = blockIdx.y * kCh, c = c0 + blockIdx.x, rows = min(kSteps, T - c * kSteps);
+  const size_t r0 = static_cast<size_t>(h0 + hd) * T + static_cast<size_t>(c) * kSteps;
+  const size_t task = static_cast<size_t>(hd) * nb + blockIdx.x;
+  const bool state = c > 0;
+  v += r0 * d;
+  out += r0 * d;
+  const float *sQ = smem + Lay::kQ, *sK = smem + Lay::kK;
+  float *sP = smem + Lay::kS;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // the row's scores and decays once (lanes the keys lane and lane + 32 it sees), then for each 32 channels:
+  // lane = channel, the keys in turn, where four or more are flagged, else a channel at a time with the lanes
+  // over the keys
+  float *s_sc = sP + (tid >> 5) * 2 * kSteps, *s_dg = s_sc + kSteps;  // the weights are consumed
+  const int t_end = min(rows, (tid >> 5) * 8 + 8);
+  for (int t = (tid >> 5) * 8; t < t_end; ++t) {
+    if (!(s_flag[t][0] | s_flag[t][1])) continue;
+    const float2 g2 = gam[t];
+    const float e0 = expf(g2.x), et = fmaf(e0, g2.y, e0), gt = g2.x + g2.y, den = s_den[t];
+    float sc[2], dg[2];
+    __syncwarp();
+#pragma unroll
+    for (int k2 = 0; k2 < 2; ++k2) {
+      const int i = lane + 32 * k2;
+      sc[k2] = 0.f;
+      dg[k2] = i <= t ? sum_diff(g2, gam[i]) : -INFINITY;
+      if (i <= t)
+        for (int f = 0; f < M; ++f) sc[k2] = fmaf(sQ[f * kLd + t], sK[f * kLd + i], sc[k2]);
+      s_sc[i] = sc[k2];
+      s_dg[i] = dg[k2];
+    }
+    __syncwarp();
+    auto read = [&](float bq, float m, float acc, float ixe, int j) {
+      return read_entry(bq, m, acc, ixe, state && bq > 0.f ? w.mu[task * dp + j] : 0.f, et, gt, den, state);
+    };
+    for (int half = 0; half < 2; ++half) {
+      unsigned fm = s_flag[t][half];
+      if (__popc(fm) >= 4) {
+        const int j = j0 + half * 32 + lane;
+        const bool on = (fm >> lane) & 1u;  // below d
+        const float bq = on ? s_b[j - j0] : 0.f;
+        const float *vc = v + (on ? j : 0);
+        float m = -INFINITY, acc = 0.f, ixe = 0.f;
+        for (int i = 0; i <= t; ++i) m = fmaxf(m, fmaf(bq, __ldg(vc + static_cast<size_t>(i) * d), s_dg[i]));
+        for (int i = 0; i <= t; ++i) {
+          const float xv = __ldg(vc + static_cast<size_t>(i) * d), y = fmaf(bq, xv, s_dg[i]);
+          const float e = bq > 0.f ? expf(y - m) : expf(s_dg[i]) * lin_value(bq, xv);
+          if (!(bq > 0.f) || y != -INFINITY) acc = fmaf(s_sc[i], e, acc);
+        }
+        if (state && on)
+          for (int f = 0; f < M; ++f) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
+        if (on) out[static_cast<size_t>(t) * d + j] = read(bq, m, acc, ixe, j);
+        continue;
+      }
+      while (fm) {
+        const int j = j0 + half * 32 + __ffs(fm) - 1;
+        fm &= fm - 1;
+        const float bq = s_b[j - j0];
+        float y[2], m = -INFINITY, acc = 0.f, ixe = 0.f;
+#pragma unroll
+        for (int k2 = 0; k2 < 2; ++k2) {
+          const int i = lane + 32 * k2;
+          const float xv = i <= t ? __ldg(v + static_cast<size_t>(i) * d + j) : 0.f;
+          y[k2] = i <= t ? fmaf(bq, xv, dg[k2]) : -INFINITY;
+          m = fmaxf(m, y[k2]);
+          if (!(bq > 0.f) && i <= t) acc = fmaf(sc[k2] * expf(dg[k2]), lin_value(bq, xv), acc);
+        }
+        if (state)
+          for (int f = lane; f < M; f += 32) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
+#pragma unroll
+        for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        if (bq > 0.f) {
+#pragma unroll
+          for (int k2 = 0; k2 < 2; ++k2)
+            if (y[k2] != -INFINITY) acc = fmaf(sc[k2], expf(y[k2] - m), acc);
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) {
+          acc += __shfl_xor_sync(0xffffffffu, acc, off);
+          ixe += __shfl_xor_sync(0xffffffffu, ixe, off);
+        }
+        if (lane == 0) out[static_cast<size_t>(t) * d + j] = read(bq, m, acc, ixe, j);
+      }
+    }
+  }
+}
+
 // LONE: the sequence is one chunk, so there is no state and the forms are found here.
 template <int M, bool LONE>
 __global__ void __launch_bounds__(kThreads, 3)
     gla_out_f32_kernel(const float *__restrict__ qf, const float *__restrict__ kf, const float *__restrict__ v,
                        const float *__restrict__ logdecay, const float *__restrict__ beta, float *__restrict__ out,
                        float *__restrict__ logz, int h0, int H, int T, int d, int dp, int c0, int nb, int vec, int vec_o,
-                       GlaWs w) {
+                       const __grid_constant__ GlaWs w) {
   using Lay = OutF32<M>;
   extern __shared__ __align__(16) float gla_smem[];
   float *sQ = gla_smem + Lay::kQ, *sK = gla_smem + Lay::kK, *sE = gla_smem + Lay::kE, *sS = gla_smem + Lay::kS, *sP = sS;
@@ -556,88 +790,11 @@ __global__ void __launch_bounds__(kThreads, 3)
       }
     }
   }
-  if (!__syncthreads_or(any)) return;
-  // ---- the flagged entries key by key, a warp per row.  The row's scores and decays once (lanes the keys
-  // lane and lane + 32 it sees), then for each 32 channels: lane = channel, the keys in turn, where four
-  // or more are flagged, else a channel at a time with the lanes over the keys.
-  float *s_sc = sP + (tid >> 5) * 2 * kSteps, *s_dg = s_sc + kSteps;  // the weights are consumed
-  const int t_end = min(rows, (tid >> 5) * 8 + 8);
-  for (int t = (tid >> 5) * 8; t < t_end; ++t) {
-    if (!(s_flag[t][0] | s_flag[t][1])) continue;
-    const float2 g2 = gam[t];
-    const float e0 = expf(g2.x), et = fmaf(e0, g2.y, e0), gt = g2.x + g2.y, den = s_den[t], lden = logf(den);
-    float sc[2], dg[2];
-    __syncwarp();
-#pragma unroll
-    for (int k2 = 0; k2 < 2; ++k2) {
-      const int i = lane + 32 * k2;
-      sc[k2] = 0.f;
-      dg[k2] = i <= t ? sum_diff(g2, gam[i]) : -INFINITY;
-      if (i <= t)
-        for (int f = 0; f < M; ++f) sc[k2] = fmaf(sQ[f * kLd + t], sK[f * kLd + i], sc[k2]);
-      s_sc[i] = sc[k2];
-      s_dg[i] = dg[k2];
-    }
-    __syncwarp();
-    // the read from the in-chunk sum acc at the shift m (linear: acc alone) and the state's part
-    auto read = [&](float bq, float m, float acc, float ixe, int j) {
-      if (!(bq > 0.f)) return lin_read(bq, (state ? fmaf(et, ixe, acc) : acc) / den);
-      const float la = acc == 0.f ? -INFINITY : m + logf(acc);
-      const float lb = ixe == 0.f ? -INFINITY : w.mu[task * dp + j] + gt + logf(ixe);
-      const float hi = fmaxf(la, lb), lo = fminf(la, lb);
-      const float ln = hi == -INFINITY ? hi : hi + log1pf(expf(lo - hi));
-      return ((la != la ? la : lb != lb ? lb : ln) - lden) / bq;
-    };
-    for (int half = 0; half < 2; ++half) {
-      unsigned fm = s_flag[t][half];
-      if (__popc(fm) >= 4) {
-        const int j = j0 + half * 32 + lane;
-        const bool on = (fm >> lane) & 1u;  // below d
-        const float bq = on ? s_b[j - j0] : 0.f;
-        const float *vc = v + r0 * d + (on ? j : 0);
-        float m = -INFINITY, acc = 0.f, ixe = 0.f;
-        for (int i = 0; i <= t; ++i) m = fmaxf(m, fmaf(bq, __ldg(vc + static_cast<size_t>(i) * d), s_dg[i]));
-        for (int i = 0; i <= t; ++i) {
-          const float xv = __ldg(vc + static_cast<size_t>(i) * d), y = fmaf(bq, xv, s_dg[i]);
-          const float e = bq > 0.f ? expf(y - m) : expf(s_dg[i]) * lin_value(bq, xv);
-          if (!(bq > 0.f) || y != -INFINITY) acc = fmaf(s_sc[i], e, acc);
-        }
-        if (state && on)
-          for (int f = 0; f < M; ++f) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
-        if (on) out[(r0 + t) * d + j] = read(bq, m, acc, ixe, j);
-        continue;
-      }
-      while (fm) {
-        const int j = j0 + half * 32 + __ffs(fm) - 1;
-        fm &= fm - 1;
-        const float bq = s_b[j - j0];
-        float y[2], m = -INFINITY, acc = 0.f, ixe = 0.f;
-#pragma unroll
-        for (int k2 = 0; k2 < 2; ++k2) {
-          const int i = lane + 32 * k2;
-          const float xv = i <= t ? __ldg(v + (r0 + i) * d + j) : 0.f;
-          y[k2] = i <= t ? fmaf(bq, xv, dg[k2]) : -INFINITY;
-          m = fmaxf(m, y[k2]);
-          if (!(bq > 0.f) && i <= t) acc = fmaf(sc[k2] * expf(dg[k2]), lin_value(bq, xv), acc);
-        }
-        if (state)
-          for (int f = lane; f < M; f += 32) ixe = fmaf(sQ[f * kLd + t], w.u[(task * M + f) * dp + j], ixe);
-#pragma unroll
-        for (int off = 16; off; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-        if (bq > 0.f) {
-#pragma unroll
-          for (int k2 = 0; k2 < 2; ++k2)
-            if (y[k2] != -INFINITY) acc = fmaf(sc[k2], expf(y[k2] - m), acc);
-        }
-#pragma unroll
-        for (int off = 16; off; off >>= 1) {
-          acc += __shfl_xor_sync(0xffffffffu, acc, off);
-          ixe += __shfl_xor_sync(0xffffffffu, ixe, off);
-        }
-        if (lane == 0) out[(r0 + t) * d + j] = read(bq, m, acc, ixe, j);
-      }
-    }
-  }
+  const int n_flagged = __syncthreads_count(any);  // threads
+  if (n_flagged > kFewFlagged)
+    read_again<M>(gla_smem, gam, s_den, s_b, s_flag, v, out, h0, T, d, dp, c0, nb, vec, w);
+  else if (n_flagged > 0)
+    read_rows<M>(gla_smem, gam, s_den, s_b, s_flag, v, out, h0, T, d, dp, c0, nb, w);
 }
 
 size_t up64(size_t x) { return (x + 63) & ~size_t(63); }
