@@ -80,22 +80,22 @@ __device__ __forceinline__ bool sample_peaked(const float *q, const float *k, co
 }
 
 // Per (b, h, channel): {beta, 1/beta (0 at 0), c, mode}: 1 linear, 0 shifted, 2 wide.  The wide
-// channels of a head also go to its list (n_wide, then the channels), their dv zeroed for the key
-// pass to add to.  From kSampleT on one more block
-// samples the head's weights; a peaked one counts as kAllWide.
-constexpr int kAllWide = 1 << 20;
+// channels of a head are also bits of its first four words (in order, so that the sums over them are
+// the same from call to call), their dv zeroed for the key pass to add to.  From kSampleT on one more
+// block samples the head's weights, and its last word marks a peaked one.
+constexpr int kWideWords = 5;
 __global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict__ q, const float *__restrict__ k,
                                                         const float *__restrict__ v, const float *__restrict__ beta,
                                                         const float *__restrict__ lse, int H, int T, int d, int causal,
-                                                        float4 *__restrict__ chan, int *__restrict__ wide,
+                                                        float4 *__restrict__ chan, unsigned *__restrict__ wide,
                                                         float *__restrict__ dv) {
   if (blockIdx.y * 32 >= d) {
     const size_t row0 = static_cast<size_t>(blockIdx.x) * T;
     const bool peak = sample_peaked(q + row0 * d, k + row0 * d, lse + row0, T, d, causal);
-    if (__syncthreads_or(peak) && threadIdx.x == 0) atomicAdd(wide + static_cast<size_t>(blockIdx.x) * (d + 1), kAllWide);
+    if (__syncthreads_or(peak) && threadIdx.x == 0) wide[blockIdx.x * kWideWords + 4] = 1u;
     return;
   }
-  __shared__ int s_wide[32];
+  __shared__ unsigned s_wide;
   __shared__ float s_mx[32][33], s_mn[32][33], s_sm[32][33];
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5, bh = blockIdx.x, j = blockIdx.y * 32 + lane;
   const float *vb = v + static_cast<size_t>(bh) * T * d;
@@ -113,27 +113,25 @@ __global__ void __launch_bounds__(1024) bwd_chan_kernel(const float *__restrict_
   s_mn[part][lane] = mn;
   s_sm[part][lane] = sm;
   __syncthreads();
-  if (part == 0 && j < d) {
+  if (part == 0) {
     for (int p = 1; p < 32; ++p) {
       mx = fmaxf(mx, s_mx[p][lane]);
       mn = fminf(mn, s_mn[p][lane]);
       sm += s_sm[p][lane];
     }
-    const float b = beta[(bh % H) * d + j], mean = sm / static_cast<float>(T), lo = mx - 3.f / b, hi = mn + 1.f / b;
+    const float b = j < d ? beta[(bh % H) * d + j] : 0.f, mean = sm / static_cast<float>(T), lo = mx - 3.f / b, hi = mn + 1.f / b;
     const bool lin = !(b > 0.f) || lo <= hi;
     const float c = lin ? (b > 0.f ? fminf(fmaxf(mean, lo), hi) : mean) : 0.5f * (mx + mn);
     // not finite (also a sum that overflowed), or too wide for the factors (e^a / beta among them)
-    const bool wd = !(fabsf(sm) < INFINITY) || !(mx - mn < INFINITY) ||
-                    !(lin || 0.5f * b * (mx - mn) + fmaxf(-logf(b), 0.f) <= kWideExp);
-    if (wd) {
-      int *list = wide + static_cast<size_t>(bh) * (d + 1);
-      list[1 + atomicAdd(list, 1) % kAllWide] = j;
-    }
-    s_wide[lane] = wd ? 1 : 0;
-    chan[static_cast<size_t>(bh) * d + j] = make_float4(b, b > 0.f ? 1.f / b : 0.f, c, wd ? 2.f : (lin ? 1.f : 0.f));
+    const bool wd = j < d && (!(fabsf(sm) < INFINITY) || !(mx - mn < INFINITY) ||
+                              !(lin || 0.5f * b * (mx - mn) + fmaxf(-logf(b), 0.f) <= kWideExp));
+    const unsigned word = __ballot_sync(0xffffffffu, wd);
+    if (lane == 0) s_wide = wide[bh * kWideWords + blockIdx.y] = word;
+    if (j < d)
+      chan[static_cast<size_t>(bh) * d + j] = make_float4(b, b > 0.f ? 1.f / b : 0.f, c, wd ? 2.f : (lin ? 1.f : 0.f));
   }
   __syncthreads();
-  if (j < d && s_wide[lane])
+  if ((s_wide >> lane) & 1u)
     for (int i = part; i < T; i += 32) dv[(static_cast<size_t>(bh) * T + i) * d + j] = 0.f;
 }
 
@@ -194,6 +192,16 @@ __device__ __forceinline__ float row_power(float m) {
   return fminf(fmaxf(__int_as_float(__float_as_int(m) & 0x7f800000), 0x1p-126f), 0x1p126f);
 }
 __device__ __forceinline__ float finite_abs(float x) { return fabsf(x) < INFINITY ? fabsf(x) : 0.f; }
+
+__device__ __forceinline__ int wide_count(const unsigned *wl) {
+  return __popc(wl[0]) + __popc(wl[1]) + __popc(wl[2]) + __popc(wl[3]);
+}
+__device__ __forceinline__ int wide_next(const unsigned *wl, int j) {  // the first wide channel after j; there is one
+  int w = ++j >> 5;
+  unsigned m = wl[w] & ~0u << (j & 31);
+  while (!m) m = wl[++w];
+  return w * 32 + __ffs(m) - 1;
+}
 
 // One wide channel's terms of a visible pair with log-weight lp, each from its own exponent:
 // q = p e^x, p expm1(x)/b and p phi(x)/b^2 with x = b (v - o).
@@ -288,7 +296,7 @@ template <int DP>
 __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
     bwd_row_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
-                   const float4 *__restrict__ chan, const int *__restrict__ wide, int *__restrict__ peaked,
+                   const float4 *__restrict__ chan, const unsigned *__restrict__ wide, int *__restrict__ peaked,
                    float *__restrict__ power, float *__restrict__ head_power, float *__restrict__ dbp,
                    float *__restrict__ dq, int T, int d, int causal, int wide_most) {
   using Lay = RowLay<DP>;
@@ -298,9 +306,9 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
         *sKn = bwd_smem + Lay::kKn, *sS = bwd_smem + Lay::kS, *sR = bwd_smem + Lay::kR, *sDb = bwd_smem + Lay::kDb;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31;
   const int rank = blockIdx.x, size = gridDim.x, bh = blockIdx.z;
-  const int *wl = wide + static_cast<size_t>(bh) * (d + 1);
-  const int n_wide = wl[0];
-  if (n_wide > wide_most) {  // pair by pair is faster, or needed
+  const unsigned *wl = wide + static_cast<size_t>(bh) * kWideWords;
+  const int n_wide = wide_count(wl);
+  if (n_wide > wide_most || wl[4]) {  // pair by pair is faster, or needed
     if (tid == 0) peaked[bh] = 1;
     return;
   }
@@ -432,8 +440,8 @@ __global__ void __launch_bounds__(256, DP <= 64 ? 2 : 1)
     }
     if (peak) peaked[bh] = 1;
     peak = peak || others != 0;
-    for (int w = 0; w < n_wide; ++w) {
-      const int j = wl[1 + w];
+    for (int w = 0, j = -1; w < n_wide; ++w) {
+      j = wide_next(wl, j);
       const float b = ch[j].x, ib = ch[j].y;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -503,7 +511,7 @@ template <int DP>
 __global__ void __launch_bounds__(256, 1)
     bwd_key_kernel(const float *__restrict__ q, const float *__restrict__ k, const float *__restrict__ v,
                    const float *__restrict__ out, const float *__restrict__ lse, const float *__restrict__ dout,
-                   const float4 *__restrict__ chan, const int *__restrict__ wide, const int *__restrict__ peaked,
+                   const float4 *__restrict__ chan, const unsigned *__restrict__ wide, const int *__restrict__ peaked,
                    const float *__restrict__ power, const float *__restrict__ head_power, float *__restrict__ dbp,
                    float *__restrict__ dk, float *__restrict__ dv, int T, int d, int causal) {
   using Lay = KeyLay<DP>;
@@ -515,8 +523,8 @@ __global__ void __launch_bounds__(256, 1)
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const int rank = blockIdx.x, size = gridDim.x, bh = blockIdx.z, k0 = static_cast<int>(blockIdx.y) * kBT;
   if (peaked[bh]) return;  // the head goes pair by pair
-  const int *wl = wide + static_cast<size_t>(bh) * (d + 1);
-  const int n_wide = wl[0];
+  const unsigned *wl = wide + static_cast<size_t>(bh) * kWideWords;
+  const int n_wide = wide_count(wl);
   const size_t base = static_cast<size_t>(bh) * T * d;
   const float4 *ch = chan + static_cast<size_t>(bh) * d;
   const bool vec = (d & 3) == 0;
@@ -614,8 +622,8 @@ __global__ void __launch_bounds__(256, 1)
       *reinterpret_cast<float4 *>(sP + row * kBT + tx * 4) =
           make_float4(pv[0] * prel, pv[1] * prel, pv[2] * prel, pv[3] * prel);
     }
-    for (int w = 0; w < n_wide; ++w) {
-      const int j = wl[1 + w];
+    for (int w = 0, j = -1; w < n_wide; ++w) {
+      j = wide_next(wl, j);
       const float b = ch[j].x, ib = ch[j].y;
       float db = 0.f;
 #pragma unroll
@@ -720,7 +728,7 @@ BwdWs bwd_ws(int BH, int T, int d) {
   w.zero_from = w.tile = w.power + static_cast<size_t>(BH) * T * sizeof(float);
   w.pairs = w.tile + n * sizeof(float);
   w.wide = w.pairs + n * sizeof(float);
-  w.peaked = w.wide + (n + BH) * sizeof(int);
+  w.peaked = w.wide + static_cast<size_t>(BH) * kWideWords * sizeof(unsigned);
   w.head_power = w.peaked + static_cast<size_t>(BH) * sizeof(int);
   w.total = w.head_power + static_cast<size_t>(BH) * sizeof(float);
   return w;
@@ -752,7 +760,8 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
   float4 *chan = reinterpret_cast<float4 *>(ws + w.chan);
   float *tile = reinterpret_cast<float *>(ws + w.tile), *power = reinterpret_cast<float *>(ws + w.power),
         *head_power = reinterpret_cast<float *>(ws + w.head_power);
-  int *wide = reinterpret_cast<int *>(ws + w.wide), *peaked = reinterpret_cast<int *>(ws + w.peaked);
+  unsigned *wide = reinterpret_cast<unsigned *>(ws + w.wide);
+  int *peaked = reinterpret_cast<int *>(ws + w.peaked);
   const int n_t = (T + kBT - 1) / kBT;
   bwd_chan_kernel<<<dim3(BH, (d + 31) / 32 + (T >= kSampleT ? 1 : 0)), 1024, 0, stream>>>(q, k, v, beta, lse, H, T, d, causal, chan, wide, dv);
   // CTAs sharing a tile: until there are about four per SM, while each has a tile of the other side
@@ -765,11 +774,11 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = launch_cluster(bwd_row_kernel<DP>, dim3(size, n_t, BH), RowLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
-                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), peaked, power, head_power, tile, dq, T, d,
+                       static_cast<const float4 *>(chan), static_cast<const unsigned *>(wide), peaked, power, head_power, tile, dq, T, d,
                        causal, wide_most);
   if (e == cudaSuccess)
     e = launch_cluster(bwd_key_kernel<DP>, dim3(size, n_t, BH), KeyLay<DP>::kBytes, stream, q, k, v, out, lse, dout,
-                       static_cast<const float4 *>(chan), static_cast<const int *>(wide), static_cast<const int *>(peaked), static_cast<const float *>(power),
+                       static_cast<const float4 *>(chan), static_cast<const unsigned *>(wide), static_cast<const int *>(peaked), static_cast<const float *>(power),
                        static_cast<const float *>(head_power), tile, dk, dv, T, d, causal);
   return e;
 }
