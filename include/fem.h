@@ -268,7 +268,7 @@ int fem_tdc_conv(const float *s, const float *u, float *h, int B, int T, int Hc,
  *   dbeta              : device, float32 [H, d], summed over batch and time
  *   1 <= d <= 256
  * fp32 on CUDA cores, O(T^2 d) like the forward.  Up to d = 128 and from T = 64 on
- * (up to 128 where the rows are few or d > 32) it allocates a small workspace (28 bytes
+ * (72 with few rows at d > 32, 96 at d > 64) it allocates a small workspace (28 bytes
  * per (b, h, channel), 4 per row) stream-ordered on `stream`, none otherwise.  dbeta is
  * summed with atomics, and from there on so is dv in channels whose beta times their
  * values' spread passes 152 or is not finite: their last bits may vary between calls.

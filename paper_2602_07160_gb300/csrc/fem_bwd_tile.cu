@@ -790,7 +790,7 @@ cudaError_t launch_tile_dp(const float *q, const float *k, const float *v, const
 // 235 / 143, T 300 3420 / 1096, d 128 T 96 740 / 592; B*H = 64 d 16 T 1024 4452 / 770.
 bool bwd_tile_takes(int B, int H, int T, int d) {
   const bool few = static_cast<long long>(B) * H * T <= kBwdFewRows;
-  const int least = d <= 32 ? 64 : d <= 64 ? (few ? 80 : 64) : (few ? 128 : 96);
+  const int least = d <= 64 ? (d > 32 && few ? 72 : 64) : 96;
   return d <= 128 && T >= least && static_cast<long long>(T) <= 64ll * 65535 && static_cast<long long>(B) * H <= 65535;
 }
 

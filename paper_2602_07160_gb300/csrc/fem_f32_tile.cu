@@ -25,8 +25,8 @@
 // what the range can drop from a sum (2^-126 of either's largest) stays below 2^-24 of an A / L of
 // kTileGuard.  An entry whose A / L is not finite or lies below that (peaked priors, wide spans,
 // infinities among the values of keys the row does not see) is summed again around its own largest
-// s_i + beta v_i, the key tiles once more (sweep_again); one of a linear channel, which only values
-// that are not finite can reject, key by key.  Every product and sum is fp32, as in fem_simt.cu.
+// s_i + beta v_i, the key tiles once more (sweep_again), or by itself (read_exact) where a warp has few;
+// likewise one of a linear channel, which only values that are not finite can reject.  Every product and sum is fp32, as in fem_simt.cu.
 //
 // Layout: two groups of 256 threads take the key tiles in turn, each with its own K, bank and P
 // tiles in shared memory and its own accumulators (the heaviest block's chain is half as long, and
@@ -52,6 +52,10 @@ constexpr float kLinTop = 3.f;
 constexpr float kTopExp = 36.f;       // largest exponent of a shifted bank
 constexpr float kWeightScale = 0x1p40f;
 constexpr float kTileGuard = 0x1p-84f;
+// What a warp evaluates one by one: its rejected entries, each counted as often as its row has 64 keys.  An
+// entry takes some 500 us at 2048 keys of 64 channels, a sweep 350 there; in a sequence's first rows a few
+// entries are common (B9 H6 T71 d64: 20.6 us, with a sweep for any 30.8).
+constexpr unsigned kFewRejected = 4;
 constexpr float kTileLag = 8.f;       // the row maximum moves when it grows by more (nats)
 
 template <int DP>
@@ -113,7 +117,7 @@ __device__ __noinline__ float read_exact(const In *qr, const In *kb, const In *v
 // The block's key tiles once more for the rejected entries of shifted channels (Lay::kAny: bit 4 c + r of a
 // thread's word is row 4 ty + r, channel chan(c)): scores as before, then in warps that have any the largest
 // s_i + beta v_i of the tile and the sum around the running one.  What bounds it is the issue of the tile's
-// (row, key, channel) terms and their exponentials.  Entry by entry, scores and all, a warp spent some 40 us on each at
+// (row, key, channel) terms and their exponentials.  Entry by entry, scores and all, a warp spends some 500 us on each at
 // T2048 d64 and peaked priors reject most of them: B1 H4 T2048 d64 causal, scores of deviation 16, beta 10 to
 // 100 73.5 ms (the warp-per-row form 2.5, with -inf for many); now 0.53 ms.
 template <typename In, int DP>
@@ -560,7 +564,7 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
     }
   }
   __syncthreads();
-  unsigned again = 0;  // entries of shifted channels to sum again: bit 4 c + r
+  unsigned rejected = 0, linear = 0;  // entries to evaluate again, those of linear channels: bit 4 c + r
   if (g == 0) {
     for (int og = 1; og < kGroups; ++og) {
       const float *st = tile_smem + DP * kTLd + og * Lay::kGroupFloats;
@@ -579,10 +583,8 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
       }
     }
     // ---- the read
-    unsigned redo[NC];  // per channel: the rows to evaluate again
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      redo[c] = 0u;
       const int j = chan(c);
       const float b = pB[j], ib = pI[j], cc = pC[j];
       const bool lin = pL[j] != 0.f;
@@ -593,10 +595,8 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
         const float x = a / l[r];
         const bool bad = lin ? !(b * x > -0.9f && fabsf(x) < INFINITY) : !(x > kTileGuard && x < INFINITY);
         if (bad && j < d && t0 + ty * 4 + r < T) {
-          if (lin)
-            redo[c] |= 1u << r;
-          else
-            again |= 1u << (4 * c + r);
+          rejected |= 1u << (4 * c + r);
+          if (lin) linear |= 1u << (4 * c + r);
         }
         if (b > 0.f) {
           // log1p(b x) or log(x), the latter as n ln 2 + log(mantissa) with ln 2 in two parts (Cody and Waite),
@@ -642,28 +642,6 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
         }
       }
     }
-    // ---- the linear channels' entries to evaluate again, one at a time by the whole warp
-    __syncwarp();  // their first values, stored by their own threads, come before lane 0's
-#pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
-      unsigned mine = 0u;
-#pragma unroll
-      for (int u = 0; u < NC; ++u) mine = u == c ? redo[u] : mine;
-      unsigned who = __ballot_sync(0xffffffffu, mine != 0u);
-      while (who) {
-        const int src = __ffs(who) - 1;
-        who &= who - 1;
-        unsigned rows = __shfl_sync(0xffffffffu, mine, src);
-        const int j = __shfl_sync(0xffffffffu, chan(c), src), ry = __shfl_sync(0xffffffffu, ty, src);
-        while (rows) {
-          const int t = t0 + ry * 4 + __ffs(rows) - 1;
-          rows &= rows - 1;
-          const float o = read_exact(qb + static_cast<size_t>(t) * d, kb, vb, causal ? t + 1 : T, d, j, pB[j], inv_sqrt_d,
-                                     lane);
-          if (lane == 0) out[(bh * T + t) * d + j] = o;
-        }
-      }
-    }
     if (tx == 0) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
@@ -671,10 +649,30 @@ __global__ void __launch_bounds__(kGroups * kGT, 1)
         sRed[(ty * 4 + r) * 2 + 1] = l[r] * (1.f / kWeightScale);
       }
     }
-    reinterpret_cast<unsigned *>(tile_smem + Lay::kAny)[gt] = again;
+    reinterpret_cast<unsigned *>(tile_smem + Lay::kAny)[gt] = rejected & ~linear;
   }
-  if (__syncthreads_or(again != 0u))
-    sweep_again<In, DP>(tile_smem, kb, vb, out + bh * T * d, T, d, t0, n_keys, causal);
+  unsigned cost = 0;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    cost += __popc(rejected & ~linear & (0x11111111u << r)) * static_cast<unsigned>(((causal ? t0 + ty * 4 + r : T - 1) >> 6) + 1);
+  const bool many = __reduce_add_sync(0xffffffffu, cost) > kFewRejected;
+  const bool sweep = __syncthreads_or(many);  // also: the rejected values are stored
+  // ---- a linear channel's entries, and others where they are few, one at a time by the whole warp
+  unsigned mine = sweep ? rejected & linear : rejected;
+  unsigned who = __ballot_sync(0xffffffffu, mine != 0u);
+  while (who) {
+    const int src = __ffs(who) - 1, sx = (src & 15) * (NC == 2 ? 2 : 4), ry = __shfl_sync(0xffffffffu, ty, src);
+    who &= who - 1;
+    unsigned bits = __shfl_sync(0xffffffffu, mine, src);
+    while (bits) {
+      const int e = __ffs(bits) - 1, c = e >> 2, t = t0 + ry * 4 + (e & 3);
+      bits &= bits - 1;
+      const int j = NC == 2 ? sx + c : (c >> 2) * 64 + sx + (c & 3);
+      const float o = read_exact(qb + static_cast<size_t>(t) * d, kb, vb, causal ? t + 1 : T, d, j, pB[j], inv_sqrt_d, lane);
+      if (lane == 0) out[(bh * T + t) * d + j] = o;
+    }
+  }
+  if (sweep) sweep_again<In, DP>(tile_smem, kb, vb, out + bh * T * d, T, d, t0, n_keys, causal);
 }
 
 template <typename In, int DP>
