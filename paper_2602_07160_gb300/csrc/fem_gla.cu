@@ -15,7 +15,8 @@
 // So is a channel whose beta is below kGlaSmallBeta and whose values stay within kGlaSmallTilt / beta: its
 // state carries expm1(beta v) / beta and o is log1p(beta ratio) / beta, since the two logarithms' rounding
 // (some 5e-7) over beta would be 0.5 at beta = 1e-6.  Its beta goes negated through the kernels, as the
-// first launch leaves it (2.5 us where no beta is that small, under the next launch's loads).
+// first launch that meets it leaves it (above kOwnForm chunks a launch of its own, 2.5 us where no beta is that
+// small).
 //
 // In chunks of 64 steps, with gamma_t the running sum of g in the chunk, three
 // launches of fp32 contractions on CUDA cores (a lone chunk needs only the last):
@@ -146,23 +147,33 @@ __device__ __forceinline__ void lin_values(float4 b, float4 (&x)[4]) {
 __device__ __noinline__ float small_read(float b, float ratio) { return log1pf(-b * ratio) / -b; }
 __device__ __forceinline__ float lin_read(float b, float ratio) { return b < 0.f ? small_read(b, ratio) : ratio; }
 
+// The forms of a block's 64 channels (all threads; a quad each): the sequence's values are read only where some
+// beta is small.
+__device__ __forceinline__ float4 sequence_forms(const float *beta, const float *vh, int h, int T, int d, int jq, int vec,
+                                                 float4 (*red)[16]) {
+  const float4 b = beta4(beta, h, d, jq);
+  float4 top = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (__syncthreads_or(maybe_small(b))) {
+#pragma unroll 4
+    for (int r = threadIdx.x >> 4; r < T; r += 16) top = abs_max(top, ld_row4(vh + static_cast<size_t>(r) * d, jq, d, vec));
+    top = max_over_rows(top, red);
+    __syncthreads();  // red is used again
+  }
+  return form_beta4(b, top);
+}
+
 // ---------------------------------------------------------------------------
-// form: block per head and 64 channels; reads the values only where some beta is small.
+// form: block per head and 64 channels, for the longer sequences: up to kOwnForm chunks every block of local
+// finds the forms itself, which spares the launch and, with a small beta, reads a sequence's values once a chunk.
 // ---------------------------------------------------------------------------
+constexpr int kOwnForm = 32;
 __global__ void __launch_bounds__(kThreads) gla_form_f32_kernel(const float *__restrict__ v, const float *__restrict__ beta,
                                                                 int h0, int H, int T, int d, int dp, int vec, GlaWs w) {
   grid_dep_launch_dependents();
   __shared__ float4 red[16][16];
-  const int tid = threadIdx.x, ty = tid >> 4, jq = blockIdx.y * kCh + (tid & 15) * 4, hd = blockIdx.x;
-  const float4 b = beta4(beta, (h0 + hd) % H, d, jq);
-  float4 top = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (__syncthreads_or(maybe_small(b))) {
-    const float *vh = v + static_cast<size_t>(h0 + hd) * T * d;
-#pragma unroll 8
-    for (int r = ty; r < T; r += 16) top = abs_max(top, ld_row4(vh + static_cast<size_t>(r) * d, jq, d, vec));
-    top = max_over_rows(top, red);
-  }
-  if (ty == 0) *reinterpret_cast<float4 *>(w.eb + static_cast<size_t>(hd) * dp + jq) = form_beta4(b, top);
+  const int jq = blockIdx.y * kCh + (threadIdx.x & 15) * 4, hd = blockIdx.x;
+  const float4 b = sequence_forms(beta, v + static_cast<size_t>(h0 + hd) * T * d, (h0 + hd) % H, T, d, jq, vec, red);
+  if (threadIdx.x < 16) *reinterpret_cast<float4 *>(w.eb + static_cast<size_t>(hd) * dp + jq) = b;
 }
 
 // ---------------------------------------------------------------------------
@@ -170,7 +181,8 @@ __global__ void __launch_bounds__(kThreads) gla_form_f32_kernel(const float *__r
 // ---------------------------------------------------------------------------
 template <int M>
 __global__ void __launch_bounds__(kThreads, 4) gla_local_f32_kernel(const float *__restrict__ kf, const float *__restrict__ v,
-                                                                 const float *__restrict__ logdecay, int h0, int T,
+                                                                 const float *__restrict__ logdecay,
+                                                                 const float *__restrict__ beta, int h0, int H, int T,
                                                                  int d, int dp, int c0, int nb, int vec, GlaWs w) {
   constexpr int RT = M / 16;  // features of a thread
   __shared__ __align__(16) float sK[kSteps * M], sE[kSteps * kCh];
@@ -198,8 +210,14 @@ __global__ void __launch_bounds__(kThreads, 4) gla_local_f32_kernel(const float 
   if (tid < kSteps) s_dg[tid] = sum_diff(gam[kSteps - 1], gam[tid]);
   if (tid == 0 && blockIdx.y == 0) w.gl[task] = gam[kSteps - 1].x;
   __syncthreads();
-  grid_dep_wait();  // eb: a dependent launch on the form kernel, which a block's loads overlap
-  const float4 b = ld4(w.eb + static_cast<size_t>(hd) * dp + jq);
+  float4 b;
+  if (T > kOwnForm * kSteps) {
+    grid_dep_wait();  // a dependent launch on the form kernel, which a block's loads overlap
+    b = ld4(w.eb + static_cast<size_t>(hd) * dp + jq);
+  } else {
+    b = sequence_forms(beta, v + static_cast<size_t>(h0 + hd) * T * d, (h0 + hd) % H, T, d, jq, vec, red);
+    if (blockIdx.x == 0 && ty == 0) *reinterpret_cast<float4 *>(w.eb + static_cast<size_t>(hd) * dp + jq) = b;
+  }
   lin_values(b, x);
   float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   float4 y[4];
@@ -856,15 +874,16 @@ cudaError_t launch_gla_m(const float *qf, const float *kf, const float *v, const
   const int vec_o = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
   for (int h0 = 0; h0 < BH; h0 += p.heads) {
     const int nh = BH - h0 < p.heads ? BH - h0 : p.heads;
-    if (n_ch > 1) gla_form_f32_kernel<<<dim3(nh, groups), kThreads, 0, stream>>>(v, beta, h0, H, T, d, dp, vec, w);
+    const bool form = n_ch > kOwnForm;
+    if (form) gla_form_f32_kernel<<<dim3(nh, groups), kThreads, 0, stream>>>(v, beta, h0, H, T, d, dp, vec, w);
     for (int c0 = 0; c0 < n_ch; c0 += p.chunks) {
       const int n = n_ch - c0 < p.chunks ? n_ch - c0 : p.chunks;
       if (n_ch > 1) {
         // the sequence's last chunk starts no other: what the scan reads in its slot goes nowhere
         const int own = c0 + n == n_ch ? n - 1 : n;
         if (own > 0)
-          e = launch_kernel(gla_local_f32_kernel<M>, dim3(own, groups, nh), dim3(kThreads), 0, stream, c0 == 0, kf, v,
-                            logdecay, h0, T, d, dp, c0, p.chunks, vec, w);
+          e = launch_kernel(gla_local_f32_kernel<M>, dim3(own, groups, nh), dim3(kThreads), 0, stream,
+                            form && c0 == 0, kf, v, logdecay, beta, h0, H, T, d, dp, c0, p.chunks, vec, w);
         if (e != cudaSuccess) return e;
         gla_scan_f32_kernel<<<dim3((M * dp + M + 255) / 256, nh), 256, 0, stream>>>(d, dp, M, c0 == 0 ? 1 : 0, n,
                                                                                     p.chunks, w);
