@@ -785,7 +785,6 @@ __global__ void __launch_bounds__(kThreads, 3)
       } else {
         flag |= !(fabsf(a) < INFINITY) ? 1u << q : 0u;
         o[q] = (state ? fmaf(et, y, a) : a) * rden;
-        if (bj[q] < 0.f) o[q] = lin_read(bj[q], o[q]);
       }
       if (jq + q >= d) flag &= ~(1u << q);
     }
@@ -806,6 +805,16 @@ __global__ void __launch_bounds__(kThreads, 3)
         atomicOr(&s_flag[t][tx >> 3], flag << ((tx & 7) * 4));
         any = true;
       }
+    }
+  }
+  if (b.x < 0.f || b.y < 0.f || b.z < 0.f || b.w < 0.f) {
+    // the small-beta channels' ratios, as stored, to their reads (in the loop above this cost 2.5 of 117 us a call)
+#pragma unroll 1
+    for (int r = 0; r < 4; ++r) {
+      float *orow = out + (r0 + ty * 4 + r) * d + jq;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (ty * 4 + r < rows && jq + q < d && bj[q] < 0.f) orow[q] = lin_read(bj[q], orow[q]);
     }
   }
   const int n_flagged = __syncthreads_count(any);  // threads
