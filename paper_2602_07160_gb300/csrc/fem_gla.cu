@@ -37,8 +37,8 @@
 // steps below kGlaFloor count as it: their weights are zero either way.
 //
 // What bounds it: instruction issue around the FMA pipe in out (three 64^3 contractions a chunk and
-// 64 channels), latency at the ends of a block.  B4 H4 T2048 m64 d128: form 2.5, local 24, scan 18, out 78 us,
-// 123 in all, against 331 for a scan that walked segments of the sequence step by step, four lanes to a
+// 64 channels), latency at the ends of a block.  B4 H4 T2048 m64 d128: local 24, scan 18, out 80 us,
+// 121 in all, against 331 for a scan that walked segments of the sequence step by step, four lanes to a
 // channel's state (passes of 90 and 229 us, one dependent step at a time); B1 H1 T64 25 against 122,
 // B4 H16 T512 m16 d32 62 against 79.  Values of ten times unit spread with beta up to 100 send most
 // entries to read_again: 354 us at the first size, 406 for the scan.
